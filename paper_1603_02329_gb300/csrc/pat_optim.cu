@@ -5,6 +5,7 @@
 //   restricted bound (Sec. V.C Eq. (constraint)), FP64 reductions and FISTA vector updates.
 // Conventions: image [Nz][Ny][Nx], x fastest; D = forward differences with a zero difference at
 // the last index of each axis; D^T its exact transpose.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -46,69 +47,147 @@ __device__ __forceinline__ void unflat(long long i, const ImgDims& D, int* c) {
 template <typename T> __device__ __forceinline__ T dfwd(const T* x, long long i, const int* c, const ImgDims& D, int a) {
     return (c[a] < D.n[a] - 1) ? x[i + D.s[a]] - x[i] : (T)0;
 }
-// (D^T q)[i] = sum_a q_a[i - s_a] [c_a >= 1] - q_a[i] [c_a <= n_a - 2]
-template <typename T>
-__device__ __forceinline__ T dT(const T* const* q, long long i, const int* c, const ImgDims& D) {
-    T v = 0;
-    for (int a = 0; a < D.d; ++a) {
-        if (c[a] >= 1) v += q[a][i - D.s[a]];
-        if (c[a] <= D.n[a] - 2) v -= q[a][i];
-    }
-    return v;
-}
+// One FGP iteration (dual of the TV prox, Sec. IV): r = q + w (q - q_prev), then
+// q_new = Pi_{|q|<=1}(r + step D x(r)) with x(r) = P_C(z - lam D^T r).
+//
+// Bound by memory: z and the last two duals read, the new one written, 1 + 3 d fields per iteration
+// (r is formed where it is read, so it is never stored).  A CTA takes a TX x TY tile of (x, y) and
+// marches along z over `chunk` planes; each plane's x(r) goes once through shared memory with a halo of
+// one column and one row, and r_z of the plane below and the plane above's x(r) stay in registers, so
+// a field is fetched from DRAM about once.  256^3 FP32: the map of 20 iterations takes 4.25 ms (0.21 ms
+// an iteration, 3.2 TB/s of the 1 + 3 d fields) against 20.2 ms for one thread per point over flat
+// indices, which formed x(r) d + 1 times from global memory, stored r, and divided 64-bit indices.
+constexpr int kFgpX = 64, kFgpY = 8;
 
-template <typename T> struct Fields3 {
-    T* f[3];
+template <typename T> struct FgpArgs {
+    int nx, ny, nz, chunk;   // chunk: planes per CTA (3-D)
+    unsigned gx, gy;         // tiles along x and y (the grid is one-dimensional: no limit on a side)
+    const T* z;
+    const T* q[3];           // q_k
+    const T* qp[3];          // q_{k-1}
+    T* qn[3];                // q_{k+1}
+    T lam, step, w;
+    int nonneg, first;       // first: q_k = q_{k-1} = 0 (not read)
 };
-template <typename T> struct CFields3 {
-    const T* f[3];
-};
 
-// x(j) = P_C(z - lam D^T r)(j)
-template <typename T>
-__device__ __forceinline__ T prox_x(const T* z, const T* const* r, long long j, const int* c, const ImgDims& D, T lam,
-                                    int nonneg) {
-    const T v = z[j] - lam * dT(r, j, c, D);
-    return nonneg ? fmax(v, (T)0) : v;
-}
+template <typename T, int D>
+__global__ void __launch_bounds__(kFgpX * kFgpY) k_fgp_iter(FgpArgs<T> A) {
+    __shared__ T sx[2][kFgpY + 1][kFgpX + 1];
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kFgpX + tx;
+    const unsigned bx = blockIdx.x % A.gx, byz = blockIdx.x / A.gx, by = byz % A.gy, bz = byz / A.gy;
+    const int x0 = bx * kFgpX, y0 = by * kFgpY;
+    const int k0 = (D == 3) ? bz * A.chunk : 0;
+    const int k1 = (D == 3) ? min(k0 + A.chunk, A.nz) : 1;
+    const int nx = A.nx, ny = A.ny;
+    const size_t sy = (size_t)nx, sz = (size_t)nx * ny;
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
 
-// One FGP iteration (dual of the TV prox, Sec. IV): q = Pi_{|q|<=1}(r + step D x(r)),
-// r_new = q + w (q - q_prev).
-template <typename T>
-__global__ void k_fgp_iter(ImgDims D, const T* z, CFields3<T> r, CFields3<T> qprev, Fields3<T> qnew, Fields3<T> rnew,
-                           T lam, T step, T w, int nonneg) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < D.N; i += (long long)gridDim.x * blockDim.x) {
-        int c[3];
-        unflat(i, D, c);
-        const T xi = prox_x(z, r.f, i, c, D, lam, nonneg);
-        T q[3];
-        T nrm2 = 0;
-        for (int a = 0; a < D.d; ++a) {
-            T g = 0;
-            if (c[a] < D.n[a] - 1) {
-                int cn[3] = {c[0], c[1], c[2]};
-                cn[a] += 1;
-                g = prox_x(z, r.f, i + D.s[a], cn, D, lam, nonneg) - xi;
+    auto r_at = [&](int a, size_t i) {
+        const T q = A.q[a][i];
+        return q + A.w * (q - A.qp[a][i]);
+    };
+    // x(r) at (x, y, k); r[] receives r_a there (0 where D_a is zero is kept by the projection), rzm
+    // is r_z of the plane below
+    auto prox = [&](int x, int y, int k, size_t i, T rzm, T* r) {
+        T v = 0;
+        if (!A.first) {
+            r[0] = r_at(0, i);
+            r[1] = r_at(1, i);
+            if (x >= 1) v += r_at(0, i - 1);
+            if (x <= nx - 2) v -= r[0];
+            if (y >= 1) v += r_at(1, i - sy);
+            if (y <= ny - 2) v -= r[1];
+            if constexpr (D == 3) {
+                r[2] = r_at(2, i);
+                if (k >= 1) v += rzm;
+                if (k <= A.nz - 2) v -= r[2];
             }
-            q[a] = r.f[a][i] + step * g;
-            nrm2 += q[a] * q[a];
+        } else {
+#pragma unroll
+            for (int a = 0; a < D; ++a) r[a] = 0;
         }
-        const T sc = (T)1 / fmax((T)1, sqrt(nrm2));
-        for (int a = 0; a < D.d; ++a) {
-            const T qa = q[a] * sc;
-            qnew.f[a][i] = qa;
-            rnew.f[a][i] = qa + w * (qa - qprev.f[a][i]);
+        v = A.z[i] - A.lam * v;
+        return A.nonneg ? fmax(v, (T)0) : v;
+    };
+
+    const int x = x0 + tx, y = y0 + ty;
+    const bool in = x < nx && y < ny;
+    // this thread's halo point, if any: the column x0 + TX (rows 0 .. TY - 1), the row y0 + TY
+    int hx = -1, hy = 0;
+    if (tid < kFgpY) {
+        hx = kFgpX;
+        hy = tid;
+    } else if (tid >= 32 && tid < 32 + kFgpX) {
+        hx = tid - 32;
+        hy = kFgpY;
+    }
+    const bool hin = hx >= 0 && x0 + hx < nx && y0 + hy < ny;
+    const size_t i0 = (size_t)y * sy + x, h0 = (size_t)(y0 + hy) * sy + (x0 + (hx < 0 ? 0 : hx));
+    T rp[3] = {0, 0, 0}, gx = 0, gy = 0, xp = 0, rzm = 0, hrzm = 0;
+    if (D == 3 && k0 >= 1 && !A.first) {
+        if (in) rzm = r_at(2, i0 + (size_t)(k0 - 1) * sz);
+        if (hin) hrzm = r_at(2, h0 + (size_t)(k0 - 1) * sz);
+    }
+    // plane k1 (3-D) only gives x(r) to plane k1 - 1's difference along z
+    const int kend = (D == 3 && k1 < A.nz) ? k1 : k1 - 1;
+    for (int k = k0; k <= kend; ++k) {
+        T r[3] = {0, 0, 0}, hr[3] = {0, 0, 0};
+        T xk = 0;
+        T(&s)[kFgpY + 1][kFgpX + 1] = sx[(k - k0) & 1];
+        if (in) xk = prox(x, y, k, i0 + (size_t)k * sz, rzm, r);
+        if (k < k1) {
+            s[ty][tx] = xk;
+            if (hin) {
+                s[hy][hx] = prox(x0 + hx, y0 + hy, k, h0 + (size_t)k * sz, hrzm, hr);
+                hrzm = hr[2];
+            }
         }
+        __syncthreads();
+        auto put = [&](int kk, const T* rr, T g0, T g1, T g2) {   // q_new of plane kk
+            T q[3] = {rr[0] + A.step * g0, rr[1] + A.step * g1, (D == 3) ? rr[2] + A.step * g2 : (T)0};
+            T nrm2 = 0;
+#pragma unroll
+            for (int a = 0; a < D; ++a) nrm2 += q[a] * q[a];
+            const T sc = (T)1 / fmax((T)1, sqrt(nrm2));
+#pragma unroll
+            for (int a = 0; a < D; ++a) A.qn[a][i0 + (size_t)kk * sz] = q[a] * sc;
+        };
+        if (in) {
+            if (D == 3 && k > k0) put(k - 1, rp, gx, gy, xk - xp);
+            if (k < k1) {
+                gx = (x < nx - 1) ? s[ty][tx + 1] - xk : (T)0;
+                gy = (y < ny - 1) ? s[ty + 1][tx] - xk : (T)0;
+                if (D == 2) put(k, r, gx, gy, (T)0);
+                else if (k == A.nz - 1) put(k, r, gx, gy, (T)0);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) rp[a] = r[a];
+        xp = xk;
+        rzm = r[2];
     }
 }
 
-template <typename T>
-__global__ void k_fgp_final(ImgDims D, const T* z, CFields3<T> q, T* x, T lam, int nonneg) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < D.N; i += (long long)gridDim.x * blockDim.x) {
-        int c[3];
-        unflat(i, D, c);
-        x[i] = prox_x(z, q.f, i, c, D, lam, nonneg);
+// x = P_C(z - lam D^T q): z and the duals read once, x written once
+template <typename T, int D>
+__global__ void __launch_bounds__(256) k_fgp_final(FgpArgs<T> A, T* x) {
+    const unsigned bx = blockIdx.x % A.gx, byz = blockIdx.x / A.gx;
+    const int i = bx * 64 + threadIdx.x, j = (byz % A.gy) * 4 + threadIdx.y, k = byz / A.gy;
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    if (i >= A.nx || j >= A.ny) return;
+    const size_t sy = (size_t)A.nx, sz = sy * A.ny, p = (size_t)k * sz + (size_t)j * sy + i;
+    T v = 0;
+    if (i >= 1) v += A.q[0][p - 1];
+    if (i <= A.nx - 2) v -= A.q[0][p];
+    if (j >= 1) v += A.q[1][p - sy];
+    if (j <= A.ny - 2) v -= A.q[1][p];
+    if constexpr (D == 3) {
+        if (k >= 1) v += A.q[2][p - sz];
+        if (k <= A.nz - 2) v -= A.q[2][p];
     }
+    v = A.z[p] - A.lam * v;
+    x[p] = A.nonneg ? fmax(v, (T)0) : v;
 }
 
 // v_a(j) = D_a y(j) / sqrt(|D y(j)|^2 + rho^2)
@@ -346,6 +425,71 @@ pat_status Ops<T>::reduce(int op, const pat_grid* g, long long n, const T* a, co
     return PAT_OK;
 }
 
+// the FGP loop: three rotating dual fields; every launch may start (programmatic dependent launch) while
+// its predecessor drains
+template <typename T, int D>
+static pat_status fgp(const ImgDims& M, const T* z, T* x, double lam, int n_inner, int nonneg, cudaStream_t s) {
+    T* buf = nullptr;
+    const size_t N = (size_t)M.N;
+    cudaError_t e = cudaMallocAsync(&buf, (size_t)3 * D * N * sizeof(T), s);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (TV prox)");
+    FgpArgs<T> A{};
+    A.nx = M.n[0];
+    A.ny = M.n[1];
+    A.nz = M.n[2];
+    A.z = z;
+    A.lam = (T)lam;
+    A.step = (T)(1.0 / (4.0 * D * lam));
+    A.nonneg = nonneg;
+    A.gx = (A.nx + kFgpX - 1) / kFgpX;
+    A.gy = (A.ny + kFgpY - 1) / kFgpY;
+    // planes per CTA: a CTA reads one plane more than it writes, so long chunks save traffic as long as
+    // about four rounds of 4 CTAs per SM remain (16 planes at 256^3); at least 4 planes
+    const long long want = 16LL * 152;
+    A.chunk = (int)std::max<long long>(4, std::min<long long>(64, (long long)A.gx * A.gy * A.nz / want));
+    const unsigned gz = (D == 3) ? (A.nz + A.chunk - 1) / A.chunk : 1;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.stream = s;
+    lc.attrs = attr;
+    auto field = [&](int k, int a) { return buf + (size_t)(k * D + a) * N; };
+    double t = 1.0, w = 0.0;   // the first iteration starts from r = q = 0
+    for (int it = 0; it < n_inner && e == cudaSuccess; ++it) {
+        for (int a = 0; a < D; ++a) {
+            A.q[a] = field(it % 3, a);
+            A.qp[a] = field((it + 2) % 3, a);
+            A.qn[a] = field((it + 1) % 3, a);
+        }
+        A.first = it == 0;
+        // after the first iteration q_0 = 0 and its extrapolation weight is (t_0 - 1) / t_1 = 0
+        if (it == 1)
+            for (int a = 0; a < D; ++a) A.qp[a] = A.q[a];
+        A.w = (T)w;
+        lc.gridDim = dim3(A.gx * A.gy * gz);
+        lc.blockDim = dim3(kFgpX, kFgpY);
+        lc.numAttrs = it == 0 ? 0 : 1;   // the first launch follows the allocation and the caller's work
+        e = cudaLaunchKernelEx(&lc, k_fgp_iter<T, D>, A);
+        const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
+        w = (t - 1.0) / tn;
+        t = tn;
+    }
+    if (e == cudaSuccess) {
+        for (int a = 0; a < D; ++a) A.q[a] = field(n_inner % 3, a);
+        A.gx = (A.nx + 63) / 64;
+        A.gy = (A.ny + 3) / 4;
+        lc.gridDim = dim3(A.gx * A.gy * (D == 3 ? A.nz : 1));
+        lc.blockDim = dim3(64, 4);
+        lc.numAttrs = 1;
+        e = cudaLaunchKernelEx(&lc, k_fgp_final<T, D>, A, x);
+    }
+    cudaFreeAsync(buf, s);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "TV prox kernels");
+    return PAT_OK;
+}
+
 template <typename T>
 pat_status Ops<T>::tv_prox(const pat_grid* g, const T* z, T* x, double lam, int n_inner, int nonneg, cudaStream_t s) {
     const ImgDims D = img_dims(*g);
@@ -354,45 +498,7 @@ pat_status Ops<T>::tv_prox(const pat_grid* g, const T* z, T* x, double lam, int 
         k_lincomb<T><<<nb, 256, 0, s>>>(D.N, x, (T)1, z, (T)0, nullptr, (T)0, nullptr, nullptr, nonneg);
         return PAT_OK;
     }
-    T* buf = nullptr;
-    const size_t fb = (size_t)D.N * sizeof(T);
-    cudaError_t e = cudaMallocAsync(&buf, 4 * 3 * fb, s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (TV prox)");
-    cudaMemsetAsync(buf, 0, 4 * 3 * fb, s);
-    T* R0[3];
-    T* R1[3];
-    T* Q0[3];
-    T* Q1[3];
-    for (int a = 0; a < 3; ++a) {
-        R0[a] = buf + (size_t)(0 * 3 + a) * D.N;
-        R1[a] = buf + (size_t)(1 * 3 + a) * D.N;
-        Q0[a] = buf + (size_t)(2 * 3 + a) * D.N;
-        Q1[a] = buf + (size_t)(3 * 3 + a) * D.N;
-    }
-    const double step = 1.0 / (4.0 * D.d * lam);
-    double t = 1.0;
-    T** r = R0;
-    T** rn = R1;
-    T** qp = Q0;
-    T** qn = Q1;
-    for (int it = 0; it < n_inner; ++it) {
-        const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
-        const double w = (t - 1.0) / tn;
-        CFields3<T> cr{{r[0], r[1], r[2]}};
-        CFields3<T> cq{{qp[0], qp[1], qp[2]}};
-        Fields3<T> fq{{qn[0], qn[1], qn[2]}};
-        Fields3<T> fr{{rn[0], rn[1], rn[2]}};
-        k_fgp_iter<T><<<nb, 256, 0, s>>>(D, z, cr, cq, fq, fr, (T)lam, (T)step, (T)w, nonneg);
-        std::swap(r, rn);
-        std::swap(qp, qn);
-        t = tn;
-    }
-    CFields3<T> cq{{qp[0], qp[1], qp[2]}};
-    k_fgp_final<T><<<nb, 256, 0, s>>>(D, z, cq, x, (T)lam, nonneg);
-    cudaFreeAsync(buf, s);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "TV prox kernels");
-    return PAT_OK;
+    return D.d == 2 ? fgp<T, 2>(D, z, x, lam, n_inner, nonneg, s) : fgp<T, 3>(D, z, x, lam, n_inner, nonneg, s);
 }
 
 template <typename T>
