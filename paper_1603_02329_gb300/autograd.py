@@ -86,15 +86,15 @@ class PATMediumFunction(torch.autograd.Function):
 def checkpoint_bytes(op: PATOperator, K: int, c2: bool = True, rho: bool = True) -> int:
     """Device memory the checkpointed sweep allocates for one call (pat_gradient_medium with interval
     K): the ceil((Nt - 1) / K) checkpoints of (u_xi, rho_xi, spectrum of p), K fields q^n for the
-    c0^2 gradient, K + 1 steps of (D+ p, D- u) and d accumulators for the rho0 gradient, and a copy
-    of the forward state."""
+    c0^2 gradient, K + 1 steps of (D+ p, D- u) and d accumulators for the rho0 gradient, a copy of
+    the forward state, and room for the adjoint's spectra between two segments (2 absorbing, else d)."""
     d = len(op.shape)
     w = 4 if op.dtype == torch.float32 else 8
     N = op.N
     nh = int(np.prod(op.shape[:-1])) * ((op.shape[-1] // 2 + 1 + 7) // 8 * 8)
     nseg = (op.Nt - 2) // K + 1 if op.Nt > 1 else 0
     b = max(nseg, 1) * (2 * d * N + 2 * nh) * w            # checkpoints
-    b += (2 * d + (1 if op.lossy else 0) + 1) * N * w + max(d, 2) * nh * 2 * w   # forward state, p0 copy
+    b += (2 * d + (1 if op.lossy else 0) + 1) * N * w + (2 if op.lossy else d) * nh * 2 * w   # forward state, p0 copy, spectra
     if c2:
         b += (1 + max(1, min(K, op.Nt))) * N * w
     if rho:

@@ -1123,7 +1123,6 @@ template <typename T> struct Plan : public PlanBase {
                                                 void* gp0_out, int K, cudaStream_t s) {
         const int Nt = H.Nt, Ns = H.Ns;
         const size_t N = (size_t)P.N, Nh = (size_t)H.nz * H.ny * H.ldh;
-        const int nspec = std::max(D, 2);
         const int nseg = (Nt > 1) ? (Nt - 2) / K + 1 : 0;    // segments of levels 1 .. Nt-1
         const size_t ck_elems = 2 * D * N + Nh * 2;           // u, rho (real) and the p spectrum
         const bool want_c2 = gc2_out != nullptr, want_rho = grho_out != nullptr;
@@ -1159,16 +1158,19 @@ template <typename T> struct Plan : public PlanBase {
             gebuf = (T*)alloc((size_t)(std::min(K, std::max(Nt - 1, 1)) + 1) * ge_slot * sizeof(T));
             ok = grho && gbx && gebuf;
         }
+        // The recomputed forward has its own u, rho and r but works on the plan's spectra, the ones the
+        // tensor maps describe, so it takes the same passes as the plain solves (128^3, per launch: D- z
+        // pass 60 -> 23 us, absorption 96 -> 20 us, y passes 20 -> 12 us against cp.async-staged 8-column
+        // kernels on spectra of its own).  The adjoint's nlive spectra that are alive between two segments
+        // wait in `live` meanwhile: two copies each per segment.
         DevPlan<T> Pf = P;
-        Pf.use_tma = 0;   // its spectra are other buffers than the tensor maps describe
+        const int nlive = P.lossy ? 2 : D;
+        cplx<T>* live = ok ? (cplx<T>*)alloc((size_t)nlive * Nh * sizeof(cplx<T>)) : nullptr;
+        ok = ok && live;
         for (int a = 0; a < D && ok; ++a) {
             ok = ok && (Pf.u[a] = (T*)alloc(N * sizeof(T))) && (Pf.rh[a] = (T*)alloc(N * sizeof(T)));
         }
         if (ok && P.lossy) ok = (Pf.rsum = (T*)alloc(N * sizeof(T))) != nullptr;
-        for (int a = 0; a < nspec && ok; ++a) {
-            ok = (Pf.spec[a] = (cplx<T>*)alloc(Nh * sizeof(cplx<T>))) != nullptr;
-            if (ok) ok = cudaMemsetAsync(Pf.spec[a], 0, Nh * sizeof(cplx<T>), s) == cudaSuccess;
-        }
         if (!ok) {
             cudaGetLastError();
             release();
@@ -1255,12 +1257,17 @@ template <typename T> struct Plan : public PlanBase {
                 for (int a = 0; a < 2 * D; ++a)
                     cudaMemcpyAsync(gebuf + (size_t)(hi - lo) * ge_slot + (size_t)a * N, gebuf + (size_t)a * N,
                                     N * sizeof(T), cudaMemcpyDeviceToDevice, s);
+            const size_t lb = Nh * sizeof(cplx<T>);
+            for (int f = 0; f < nlive && j < nseg - 1; ++f)
+                cudaMemcpyAsync(live + (size_t)f * Nh, P.spec[f], lb, cudaMemcpyDeviceToDevice, s);
             restore(j);
             for (int n = lo; n < hi; ++n) {
                 DevPlan<T> Q = Pf;
                 fwd_hooks(Q, n - lo);
                 fwd_step_on<D>(Q, n, junk, qbuf ? qbuf + (size_t)(n - lo) * N : (T*)nullptr, s);
             }
+            for (int f = 0; f < nlive && j < nseg - 1; ++f)
+                cudaMemcpyAsync(P.spec[f], live + (size_t)f * Nh, lb, cudaMemcpyDeviceToDevice, s);
             int top = hi;
             if (hi == Nt - 1) {
                 DevPlan<T> Q = adj_hooks(Nt - 1, lo);   // lossless tail: density part of step Nt - 2
