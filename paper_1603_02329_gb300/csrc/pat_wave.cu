@@ -12,6 +12,7 @@
 #include <type_traits>
 
 #include "pat_host.h"
+#include "pat_mx.h"
 #include "pat_persist.cuh"
 #include "pat_p2.h"
 #include "pat_smooth.h"
@@ -348,7 +349,8 @@ template <typename T> struct Plan : public PlanBase {
             rowu1_pin = (ul >= 2 && ul <= 32 && (ul & (ul - 1)) == 0) ? ul : 0;
             info.rowu1 = use_rowu1 ? 1 : 0;
         }
-        row_smem = row_smem_bytes<T>(D, h.nx, h.ldh, cfg.row_lines);
+        CHK2(build_mx(h));
+        row_smem = row_smem_bytes<T>(D, h.nx, h.ldh, gen_lines());
         row2_smem = use_row2 ? row2_layout<T>(D, h.nx, h.ldh, cfg.row_lines).bytes : 0;
         spec_smem = spec_bytes(D, std::max(h.ny, h.nz), cfg.col_w);
         if (count_only) return PAT_OK;
@@ -366,8 +368,9 @@ template <typename T> struct Plan : public PlanBase {
         cudaError_t e = cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamCreate");
         CHK2(build_kap());
+        CHK2(build_mx_tables());
         CHK2(configure_persistent(h));
-        info.layout[0] = persistent ? pcfg.W : cfg.col_w;
+        info.layout[0] = persistent ? pcfg.W : (use_mx_spec ? mx_w : cfg.col_w);
         info.layout[1] = persistent ? pcfg.ppc : cfg.row_lines;
         if (!persistent) {
             st = (D == 2) ? tune_graph<2>() : tune_graph<3>();
@@ -375,6 +378,119 @@ template <typename T> struct Plan : public PlanBase {
         }
         info.spec_chunks = (!persistent && D == 3) ? chunk_count() : 1;
         return PAT_OK;
+    }
+
+    // ---------------------------------------------------------------------------------------
+    // mixed-radix per-phase kernels (pat_mx.cuh)
+    // ---------------------------------------------------------------------------------------
+    bool use_mx_row = false, use_mx_spec = false;
+    MxAxis mxa[3] = {};
+    const cplx<T>* mxt[3] = {nullptr, nullptr, nullptr};   // their twiddle tables
+    T* mx_kap = nullptr;   // kappa / N, [outer][line][ldh]
+    const double* mx_kv[3] = {nullptr, nullptr, nullptr};
+    T* mx_abs = nullptr;   // |k|^(y-2) / N and |k|^(y-1) / N, [2][outer][line][ldh] (absorbing plans)
+    int mx_w = 1;          // columns per spectral CTA
+    int optin_smem = 0;
+
+    // Lines that are no power of two take these kernels where a schedule exists, and so do all lines of FP32
+    // 2-D plans (their per-phase kernels run in batches and gradients, untuned: the batch of eight uneven
+    // instances takes 43.2 ms with them and 47.4 ms with k_row2 / k_spec2 for its 256^2 instances) and of
+    // double 3-D plans (64^3: 418 against 588 us a step, 80 x 96 x 128: 1182 against 1343).  FP32 3-D and
+    // double 2-D plans keep k_row2 / k_spec2 on power-of-two lines (64^3 FP32: 59 against 72 us; 256^2
+    // double: 210 against 283).  PAT_MX=0: none, 2: every line.
+    pat_status build_mx(const HostTables& h) {
+        const char* ev = std::getenv("PAT_MX");
+        const int mode = ev ? std::atoi(ev) : 1;
+        if (mode == 0 || arena || count_only) return PAT_OK;
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&optin_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        const int D = h.d, n[3] = {h.nx, h.ny, h.nz};
+        bool ok[3] = {};
+        for (int a = 0; a < D; ++a) ok[a] = mx_axis(n[a], mx_r1max<T>(), 0, &mxa[a]);
+        const bool all = mode == 2 || (D == 2) == (sizeof(T) == 4);
+        use_mx_row = ok[0] && (all || !use_row2) && mx_row_fits(2);
+        use_mx_spec = ok[1] && (D == 2 || ok[2]) && (all || !use_spec2) && mx_spec_fits(1);
+        pat_status st = PAT_OK;
+        for (int a = 0; a < D; ++a) {
+            if (!(a == 0 ? use_mx_row : use_mx_spec)) continue;
+            mxt[a] = upload_c(mx_table(h.tw[a], mxa[a]), &st);
+            if (!mxt[a]) return st;
+        }
+        if (use_mx_spec) {
+            const size_t nt = (size_t)h.ny * h.nz * h.ldh;
+            for (int a = 0; a < D; ++a)
+                if (!(mx_kv[a] = upload<double>(h.kv[a], &st))) return st;
+            mx_kap = dalloc<T>(nt, &st);
+            if (!mx_kap) return st;
+            if (h.lossy && !(mx_abs = dalloc<T>(2 * nt, &st))) return st;
+        }
+        // before (or without) the tuner, which a plan with a persistent kernel does not run: 8 lines and 4
+        // columns per CTA (the batch: 43.2 ms; 4 lines 43.7, 16 lines 48.7; 2 lines and 2 columns 59.2)
+        if (use_mx_row && !(std::getenv("PAT_ROW_LINES") && mx_row_fits(cfg.row_lines)))
+            for (int r : {8, 4, 2}) {
+                cfg.row_lines = r;
+                if (P.nlines % r == 0 && mx_row_fits(r)) break;
+            }
+        if (use_mx_spec) {
+            mx_w = std::getenv("PAT_COL_W") ? cfg.col_w : 4;
+            while (mx_w > 1 && !mx_spec_fits(mx_w)) mx_w /= 2;
+        }
+        return PAT_OK;
+    }
+    bool mx_row_fits(int r) const {
+        for (int k = R2_FWD_U; k <= R2_ADJ_P; ++k)
+            if (mx_row_smem<T>(H.d, k, P.lossy, 1, mxa[0], r) > (size_t)optin_smem) return false;
+        return true;
+    }
+    bool mx_spec_fits(int w) const {
+        for (int a = 1; a < H.d; ++a)
+            if (mx_spec_smem<T>(H.d, SPEC_GRADT, mxa[a], w) > (size_t)optin_smem ||
+                mx_spec_smem<T>(H.d, SPEC_GRAD, mxa[a], w) > (size_t)optin_smem)
+                return false;
+        return true;
+    }
+    pat_status build_mx_tables() {
+        if (!mx_kap) return PAT_OK;
+        const MxTableArgs A{H.d, H.ny, H.nz, H.nxh, H.ldh, {mx_kv[0], mx_kv[1], mx_kv[2]}, H.kap_a, H.pha, H.phb, H.invN};
+        cudaError_t e = mx_tables<T>(A, mx_kap, mx_abs, cap_stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(cap_stream);
+        return e == cudaSuccess ? PAT_OK : cuda_fail(e, "multiplier tables");
+    }
+    void mx_row(int kind, const DevPlan<T>& Q, cudaStream_t s, int flag, T* data_row, const T* h_row, T* qrow, T* gc2,
+                const T* p0c) {
+        const int D = Q.d, R = cfg.row_lines;
+        const bool u = kind == R2_FWD_U || kind == R2_ADJ_U;
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(P.nlines / R, u ? D : 1);
+        lc.blockDim = dim3(mx_row_threads(mxa[0], mx_row_dims(D, kind, Q.lossy, Q.atd).nb, R));
+        lc.dynamicSmemBytes = mx_row_smem<T>(D, kind, Q.lossy, Q.atd, mxa[0], R);
+        lc.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+        note_launch(D == 2 ? mx_row_launch_d<T, 2>(&lc, kind, Q, mxa[0], mxt[0], R, flag, data_row, h_row, qrow, gc2, p0c)
+                           : mx_row_launch_d<T, 3>(&lc, kind, Q, mxa[0], mxt[0], R, flag, data_row, h_row, qrow, gc2, p0c));
+    }
+    // F: fields of a plain transform; the absorption tables hold no time-reversal window
+    void mx_spec(int mode, const DevPlan<T>& Q, cudaStream_t s, int lax, int F) {
+        const int D = Q.d, W = mx_w;
+        const bool one = mode == SPEC_GRAD || mode == SPEC_GRADT;
+        const int fields = one ? 1 : (mode == SPEC_ABS ? 2 : (mode == SPEC_PLAIN_FWD || mode == SPEC_PLAIN_INV ? F : D));
+        const T* mt = mode != SPEC_ABS ? mx_kap : (Q.tr_kc2 > (T)0 ? nullptr : mx_abs);
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(fields, (Q.nxh + W - 1) / W, lax == 1 ? Q.nz : Q.ny);
+        lc.blockDim = dim3(mx_spec_threads(mxa[lax], W));
+        lc.dynamicSmemBytes = mx_spec_smem<T>(D, mode, mxa[lax], W);
+        lc.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+        note_launch(mx_spec_launch<T>(&lc, D, mode, Q, mxa[lax], mxt[lax], W, lax, mt));
     }
 
     bool use_zreg = false;
@@ -522,20 +638,29 @@ template <typename T> struct Plan : public PlanBase {
         std::vector<int> chunk_cands{spec_chunks};
         if (D == 3 && !std::getenv("PAT_SPEC_CHUNKS")) chunk_cands = {1, 2, 4, 8};
         int best_chunks = spec_chunks;
+        if (use_mx_spec) {   // no radix schedules, no chunks
+            scheds = {P.spec16};
+            chunk_cands = {1};
+        }
+        int best_mxw = mx_w;
+        std::vector<int> widths{1, 2, 4, 8};
+        if (use_mx_spec && sizeof(T) == 4) widths.push_back(16);
         for (int nchunk : chunk_cands)
         for (int sched : scheds)
-        for (int w : {1, 2, 4, 8}) {
+        for (int w : widths) {
             if (fw && w != base.col_w) continue;
-            if (sizeof(T) == 8 && w > 4) continue;
+            if (sizeof(T) == 8 && w > (use_mx_spec ? 8 : 4)) continue;
             for (int r : {2, 4, 8, 16}) {
                 if (fr && r != base.row_lines) continue;
                 if (P.nlines % r != 0) continue;
+                if ((use_mx_row && !mx_row_fits(r)) || (use_mx_spec && !mx_spec_fits(w))) continue;
                 LaunchCfg c = base;
-                c.col_w = w;
+                c.col_w = use_mx_spec ? base.col_w : w;
                 c.row_lines = r;
                 c.col_threads = std::min(256, std::max(64, (D * w * L / 8 + 31) / 32 * 32));
-                if (!tile_fits(w)) continue;
-                const size_t rs = row_smem_bytes<T>(D, H.nx, H.ldh, r), ss = spec_bytes(D, L, w);
+                if (!use_mx_spec && !tile_fits(w)) continue;
+                const size_t rs = row_smem_bytes<T>(D, H.nx, H.ldh, use_mx_row ? 2 : r), ss = spec_bytes(D, L, c.col_w);
+                mx_w = w;
                 const size_t r2 = use_row2 ? row2_layout<T>(D, H.nx, H.ldh, r).bytes : 0;
                 if (r2 > (size_t)optin) continue;
                 if (rs > (size_t)optin || ss + 64 > (size_t)optin) continue;   // 64: the spectral kernels' static mbarrier
@@ -560,17 +685,19 @@ template <typename T> struct Plan : public PlanBase {
                     best = c;
                     best_sched = sched;
                     best_chunks = nchunk;
+                    best_mxw = w;
                 }
             }
         }
         cudaError_t e = take_launch_err();
         if (e != cudaSuccess) return cuda_fail(e, "autotune (per-phase kernels)");
         cfg = best;
+        mx_w = best_mxw;
         P.spec16 = best_sched;
         info.schedule = P.spec16;
         spec_chunks = best_chunks;
         info.spec_chunks = chunk_count();
-        row_smem = row_smem_bytes<T>(D, H.nx, H.ldh, cfg.row_lines);
+        row_smem = row_smem_bytes<T>(D, H.nx, H.ldh, gen_lines());
         row2_smem = use_row2 ? row2_layout<T>(D, H.nx, H.ldh, cfg.row_lines).bytes : 0;
         spec_smem = spec_bytes(D, L, cfg.col_w);
         // the timed steps left arbitrary values in the work buffers; the solves re-initialise the
@@ -579,7 +706,7 @@ template <typename T> struct Plan : public PlanBase {
         for (int a = 0; a < std::max(D, 2); ++a) cudaMemsetAsync(P.spec[a], 0, Nh * sizeof(cplx<T>), cap_stream);
         e = cudaStreamSynchronize(cap_stream);
         if (e != cudaSuccess) return cuda_fail(e, "autotune");
-        info.layout[0] = cfg.col_w;
+        info.layout[0] = use_mx_spec ? mx_w : cfg.col_w;
         info.layout[1] = cfg.row_lines;
         info.tuned = tried > 1;
         return PAT_OK;
@@ -780,6 +907,8 @@ template <typename T> struct Plan : public PlanBase {
         seta((const void*)k_spec<T, D, SPEC_GRADT>, spec_smem);
         if (e == cudaSuccess && use_spec2) e = spec2_set_attrs<T>(optin);
         if (e == cudaSuccess && use_row2) e = row2_set_attrs<T>(optin);
+        if (e == cudaSuccess && use_mx_row) e = D == 2 ? mx_row_attrs_d<T, 2>(optin) : mx_row_attrs_d<T, 3>(optin);
+        if (e == cudaSuccess && use_mx_spec) e = mx_spec_attrs<T>(optin);
         if constexpr (std::is_same<T, float>::value) {
             if (e == cudaSuccess && use_rowu1) e = rowu1_set_attrs(optin);
         }
@@ -809,6 +938,10 @@ template <typename T> struct Plan : public PlanBase {
     void row_launch(int kind, const DevPlan<T>& Q, cudaStream_t s, int flag, T* data_row = nullptr,
                     const T* h_row = nullptr, T* qrow = nullptr, T* gc2 = nullptr, const T* p0c = nullptr) {
         const int R = cfg.row_lines, G = row_grid(), B = cfg.row_threads;
+        if (use_mx_row) {
+            mx_row(kind, Q, s, flag, data_row, h_row, qrow, gc2, p0c);
+            return;
+        }
         if constexpr (std::is_same<T, float>::value) {
             if (use_rowu1 && D == 3 && (kind == R2_FWD_U || kind == R2_ADJ_U)) {
                 cudaLaunchConfig_t lc = {};
@@ -857,6 +990,9 @@ template <typename T> struct Plan : public PlanBase {
     // launch helpers (used while capturing, or directly on a stream)
     // ---------------------------------------------------------------------------------------
     int row_grid() const { return P.nlines / cfg.row_lines; }
+    // x-lines per CTA of the generic row kernels: the initial states and end steps of the solves run in
+    // them whatever the step's row kernels are
+    int gen_lines() const { return use_mx_row ? 2 : cfg.row_lines; }
 
     // The launchers of the power-of-two kernels return an error without touching CUDA's last-error
     // state when they have no kernel for the request; the first such error is kept here and
@@ -893,7 +1029,7 @@ template <typename T> struct Plan : public PlanBase {
     // chunk's intermediate spectra can stay in L2 between the passes (1 = all tiles at once)
     int spec_chunks = 1;
     int spec_tiles() const { return (P.nxh + cfg.col_w - 1) / cfg.col_w; }
-    int chunk_count() const { return std::max(1, std::min(spec_chunks, spec_tiles())); }
+    int chunk_count() const { return use_mx_spec ? 1 : std::max(1, std::min(spec_chunks, spec_tiles())); }
 
     template <int D, int MODE> void spec_launch(cudaStream_t s, int lax, int F, int t0 = 0, int nt = 0) {
         spec_launch_on<D, MODE>(P, s, lax, F, t0, nt);
@@ -901,6 +1037,10 @@ template <typename T> struct Plan : public PlanBase {
     // tiles t0 .. t0 + nt - 1 (nt = 0: all)
     template <int D, int MODE>
     void spec_launch_on(const DevPlan<T>& Q0, cudaStream_t s, int lax, int F, int t0 = 0, int nt = 0) {
+        if (use_mx_spec) {
+            mx_spec(MODE, Q0, s, lax, F);
+            return;
+        }
         DevPlan<T> Q = Q0;
         Q.tile0 = t0;
         const int tiles = nt > 0 ? nt : (Q.nxh + cfg.col_w - 1) / cfg.col_w;
@@ -1199,7 +1339,7 @@ template <typename T> struct Plan : public PlanBase {
                 return sst;
             }
         }
-        const int R = cfg.row_lines, G = row_grid(), B = cfg.row_threads;
+        const int R = gen_lines(), G = P.nlines / R, B = cfg.row_threads;
         auto save = [&](int j) {
             T* c = ckpt + (size_t)j * ck_elems;
             for (int a = 0; a < D; ++a) {
@@ -1379,7 +1519,7 @@ template <typename T> struct Plan : public PlanBase {
         if (st != PAT_OK) return st;
         const int Nt = H.Nt, Ns = H.Ns;
         const size_t N = (size_t)P.N;
-        const int R = cfg.row_lines, G = row_grid(), B = cfg.row_threads;
+        const int R = gen_lines(), G = P.nlines / R, B = cfg.row_threads;
         T* junk = aux_rows;   // gathered samples of the solve (not used)
         cudaError_t e = cudaMemcpyAsync(P.data, data, (size_t)Nt * Ns * sizeof(T), cudaMemcpyDefault, s);
         for (int a = 0; a < D && e == cudaSuccess; ++a) e = cudaMemsetAsync(P.u[a], 0, N * sizeof(T), s);
@@ -1422,7 +1562,7 @@ template <typename T> struct Plan : public PlanBase {
         if (st != PAT_OK) return st;
         const int Nt = H.Nt, Ns = H.Ns;
         const size_t N = (size_t)P.N, Nh = (size_t)H.nz * H.ny * H.ldh;
-        const int R = cfg.row_lines, G = row_grid(), B = cfg.row_threads;
+        const int R = gen_lines(), G = P.nlines / R, B = cfg.row_threads;
         T* junk = aux_rows + (size_t)std::max(Nt - 1, 1) * std::max(Ns, 1);
         cudaError_t e = cudaMemcpyAsync(P.data, resid, (size_t)Nt * Ns * sizeof(T), cudaMemcpyDefault, s);
         if (e != cudaSuccess) return cuda_fail(e, "copy residual");
@@ -1511,7 +1651,7 @@ template <typename T> struct Plan : public PlanBase {
     }
 
     template <int D> void record_forward(cudaStream_t s) {
-        const int R = cfg.row_lines, G = row_grid(), B = cfg.row_threads;
+        const int R = gen_lines(), G = P.nlines / R, B = cfg.row_threads;
         const int Nt = H.Nt, Ns = H.Ns;
         probe_next = 0;
         probe_names[0].clear();
@@ -1538,7 +1678,7 @@ template <typename T> struct Plan : public PlanBase {
     }
 
     template <int D> void record_adjoint(cudaStream_t s) {
-        const int R = cfg.row_lines, G = row_grid(), B = cfg.row_threads;
+        const int R = gen_lines(), G = P.nlines / R, B = cfg.row_threads;
         const int Nt = H.Nt, Ns = H.Ns;
         const size_t N = (size_t)P.N;
         for (int a = 0; a < D; ++a) {
