@@ -85,7 +85,7 @@ typedef struct {
     double dt;
     double c_ref;       /* max sound speed (kappa correction, PML scaling) */
     int path;           /* 0: CUDA graph of per-phase kernels; 1: one persistent kernel per solve;
-                           2: the same, register-fused transforms (power-of-two 2-D grids) */
+                           2: the same on power-of-two 2-D grids (FP32: register-fused transforms) */
     int layout[2];      /* launch layout: path 0 -> columns per spectral CTA, x-lines per row CTA;
                            paths 1, 2 -> columns per CTA, x-line pairs per CTA */
     int tuned;          /* 1 when the layout was chosen by timing the feasible candidates */

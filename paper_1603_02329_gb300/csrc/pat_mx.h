@@ -7,6 +7,7 @@
 #include <vector>
 
 #include <algorithm>
+#include <cmath>
 
 #include "pat_p2.h"
 
@@ -36,6 +37,9 @@ inline unsigned mx_magic(int d) { return d == 1 ? 0u : (unsigned)(((1ull << 32) 
 //   largest radix.  Radices stay small on purpose: the outer stages are unrolled code that every warp runs
 //   once per launch, and with radices up to 16 (two stages for most lines up to 256) the kernels waited for
 //   instructions (4 to 9 stall cycles per issue, 128 registers).
+//   stage > 0 (the persistent kernel): the least work of one thread over all stages, where the last stage
+//   counts twice (its threads run two butterflies) and a third stage costs `stage`.  With a butterfly or
+//   less per thread a phase takes as long as its longest threads.
 inline bool mx_axis(int n, int r1max, int stage, MxAxis* out) {
     int best = 1 << 30;
     MxAxis a{};
@@ -87,6 +91,46 @@ inline std::vector<std::complex<double>> mx_table(const std::vector<std::complex
             for (int b = 0; b < a.R0 * a.RL; ++b)
                 t.push_back(tw[(size_t)((b % a.RL) + a.RL * r) * (b / a.RL) % a.n]);
     return t;
+}
+
+// Mean gain, less 1, of a forward and an inverse transform of an axis whose twiddles and butterfly constants
+// are rounded to T: the mean of |fl(w)|^2 - 1 over the factors that an element meets.  It is the same for
+// every step (a few 1e-8 in FP32), so kappa / N is divided by it.
+template <typename T> double mx_unit(std::complex<double> w) {
+    const double c = (double)(T)w.real(), s = (double)(T)w.imag();
+    return c * c + s * s - 1.0;
+}
+template <typename T> double mx_radix_gain(int R) {
+    const auto w = [](int m, int n) { return std::polar(1.0, 2.0 * M_PI * m / n); };
+    switch (R) {
+        case 8: case 16: {   // even / odd split: the odd half meets the twiddles
+            double g = 0.0;
+            for (int k = 0; k < R / 2; ++k) g += mx_unit<T>(w(k, R)) / R;
+            return g + (R == 16 ? mx_radix_gain<T>(8) : 0.0);
+        }
+        case 9: {
+            double g = 0.0;
+            for (int k = 0; k < 9; ++k) g += mx_unit<T>(w((k / 3) * (k % 3), 9)) / 9.0;
+            return g + 2.0 * mx_radix_gain<T>(3);
+        }
+        case 6: case 12: return mx_radix_gain<T>(3);
+        case 10: return mx_radix_gain<T>(5);
+        case 14: return mx_radix_gain<T>(7);
+        case 15: return mx_radix_gain<T>(3) + mx_radix_gain<T>(5);
+        case 3: case 5: case 7: {
+            double g = 0.0;
+            for (int k = 0; k < R; ++k)
+                for (int r = 0; r < R; ++r) g += mx_unit<T>(w(k * r % R, R)) / (R * R);
+            return g;
+        }
+        default: return 0.0;   // 2, 4: exact
+    }
+}
+template <typename T> double mx_gain(const MxAxis& a, const std::vector<std::complex<double>>& table) {
+    double last = 0.0, mid = 0.0;
+    const size_t nl = (size_t)(a.RL - 1) * a.M;
+    for (size_t i = 0; i < table.size(); ++i) (i < nl ? last : mid) += mx_unit<T>(table[i]);
+    return (last + mid) / a.n + mx_radix_gain<T>(a.R0) + (a.R1 > 1 ? mx_radix_gain<T>(a.R1) : 0.0) + mx_radix_gain<T>(a.RL);
 }
 
 template <typename T> constexpr int mx_r1max() { return sizeof(T) == 4 ? 16 : 10; }
@@ -141,7 +185,22 @@ struct MxTableArgs {
     int d, ny, nz, nxh, ldh;
     const double* kv[3];   // wavenumbers per axis (device)
     double kap_a, pha, phb, invN;
+    double scale;          // of kappa: takes out mean rounding errors (k_mx_kap)
 };
 template <typename T> cudaError_t mx_tables(const MxTableArgs& A, T* kap, T* abs, cudaStream_t s);
+
+// ---- the persistent 2-D solve on these stages (pat_pmx.cuh) ----
+template <typename T> const void* pmx_kernel(bool adjoint);
+template <typename T> size_t pmx_smem(const MxAxis& x, const MxAxis& y, const PersistCfg& c, int lossy);
+template <typename T>
+cudaError_t pmx_launch(bool adjoint, const cudaLaunchConfig_t* lc, const DevPlan<T>& P, const PersistCfg& C,
+                       const MxAxis& x, const MxAxis& y, const cplx<T>* twx, const cplx<T>* twy, const T* kap,
+                       const T* abs, unsigned* gbar);
+// threads: a stage-0 butterfly of its line pairs or columns each
+inline int pmx_threads(const MxAxis& x, const MxAxis& y, int ppc, int W) {
+    const int rowt = 2 * ppc * std::max(x.m0, x.M);
+    const int colt = 2 * W * std::max(y.m0, y.M);
+    return std::min(256, std::max(128, (std::max(rowt, colt) + 31) / 32 * 32));
+}
 
 }  // namespace pat

@@ -383,10 +383,14 @@ template <typename T> struct Plan : public PlanBase {
     // ---------------------------------------------------------------------------------------
     // mixed-radix per-phase kernels (pat_mx.cuh)
     // ---------------------------------------------------------------------------------------
-    bool use_mx_row = false, use_mx_spec = false;
+    bool use_mx_row = false, use_mx_spec = false, mx_2d = false;
     MxAxis mxa[3] = {};
     const cplx<T>* mxt[3] = {nullptr, nullptr, nullptr};   // their twiddle tables
+    MxAxis pxa[2] = {};                                    // schedules and tables of the persistent kernel
+    const cplx<T>* pxt[2] = {nullptr, nullptr};
     T* mx_kap = nullptr;   // kappa / N, [outer][line][ldh]
+    T* px_kap = nullptr;   // the same for the persistent kernel's schedules
+    double mx_gain_sum = 0.0, px_gain = 0.0;
     const double* mx_kv[3] = {nullptr, nullptr, nullptr};
     T* mx_abs = nullptr;   // |k|^(y-2) / N and |k|^(y-1) / N, [2][outer][line][ldh] (absorbing plans)
     int mx_w = 1;          // columns per spectral CTA
@@ -411,18 +415,29 @@ template <typename T> struct Plan : public PlanBase {
         const bool all = mode == 2 || (D == 2) == (sizeof(T) == 4);
         use_mx_row = ok[0] && (all || !use_row2) && mx_row_fits(2);
         use_mx_spec = ok[1] && (D == 2 || ok[2]) && (all || !use_spec2) && mx_spec_fits(1);
+        mx_2d = D == 2 && ok[0] && ok[1];   // the any-length persistent kernel
         pat_status st = PAT_OK;
         for (int a = 0; a < D; ++a) {
+            if (mx_2d) {
+                mx_axis(n[a], mx_r1max<T>(), sizeof(T) == 4 ? 8 : 4, &pxa[a]);
+                const auto t = mx_table(h.tw[a], pxa[a]);
+                px_gain += mx_gain<T>(pxa[a], t);
+                pxt[a] = upload_c(t, &st);
+                if (!pxt[a]) return st;
+            }
             if (!(a == 0 ? use_mx_row : use_mx_spec)) continue;
-            mxt[a] = upload_c(mx_table(h.tw[a], mxa[a]), &st);
+            const auto t = mx_table(h.tw[a], mxa[a]);
+            mx_gain_sum += mx_gain<T>(mxa[a], t);
+            mxt[a] = upload_c(t, &st);
             if (!mxt[a]) return st;
         }
-        if (use_mx_spec) {
+        if (use_mx_spec || mx_2d) {
             const size_t nt = (size_t)h.ny * h.nz * h.ldh;
             for (int a = 0; a < D; ++a)
                 if (!(mx_kv[a] = upload<double>(h.kv[a], &st))) return st;
             mx_kap = dalloc<T>(nt, &st);
             if (!mx_kap) return st;
+            if (mx_2d && !(px_kap = dalloc<T>(nt, &st))) return st;
             if (h.lossy && !(mx_abs = dalloc<T>(2 * nt, &st))) return st;
         }
         // before (or without) the tuner, which a plan with a persistent kernel does not run: 8 lines and 4
@@ -452,8 +467,29 @@ template <typename T> struct Plan : public PlanBase {
     }
     pat_status build_mx_tables() {
         if (!mx_kap) return PAT_OK;
-        const MxTableArgs A{H.d, H.ny, H.nz, H.nxh, H.ldh, {mx_kv[0], mx_kv[1], mx_kv[2]}, H.kap_a, H.pha, H.phb, H.invN};
+        MxTableArgs A{H.d, H.ny, H.nz, H.nxh, H.ldh, {mx_kv[0], mx_kv[1], mx_kv[2]}, H.kap_a, H.pha, H.phb, H.invN, 1.0};
+        double dts = 1.0, gm = 0.0, gp = 0.0;
+        if (sizeof(T) == 4) {   // in double such errors are below the transforms' own
+            // dt, and the medium's mean rounding error (of a homogeneous one, the same at every point): kappa
+            // scales D+ and D-, so it takes half of that of b rho0 c0^2
+            const size_t N = (size_t)P.N, step = std::max<size_t>(1, N >> 20);
+            double med = 0.0;
+            size_t cnt = 0;
+            const auto err = [](double v) { return (double)(T)v / v - 1.0; };
+            for (size_t i = 0; i < N; i += step, ++cnt) {
+                for (int a = 0; a < H.d; ++a) med += err(H.b[a][i]) / H.d;
+                med += err(H.rho0[i]) + err(H.c2[i]);
+            }
+            dts = H.dt / (double)(T)H.dt / (1.0 + 0.5 * med / (double)cnt);
+            gm = mx_gain_sum;
+            gp = px_gain;
+        }
+        A.scale = dts / (1.0 + gm);
         cudaError_t e = mx_tables<T>(A, mx_kap, mx_abs, cap_stream);
+        if (e == cudaSuccess && px_kap) {
+            A.scale = dts / (1.0 + gp);
+            e = mx_tables<T>(A, px_kap, nullptr, cap_stream);
+        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(cap_stream);
         return e == cudaSuccess ? PAT_OK : cuda_fail(e, "multiplier tables");
     }
@@ -718,6 +754,33 @@ template <typename T> struct Plan : public PlanBase {
     PersistCfg pcfg{};
     int persist_threads = 256;
     bool persist_p2 = false;
+    bool persist_mx = false;   // the any-length persistent kernel (pat_pmx.cuh) runs the solves
+
+    // a launch layout of a persistent kernel: columns and line pairs per CTA, grid, threads, shared memory
+    struct PersistLayout {
+        PersistCfg c;
+        int G, threads;
+        size_t smem;
+    };
+    PersistLayout rev{};       // of k_pmx for time reversal (G = 0: not available)
+
+    PersistLayout persist_layout(int W, int ppc, bool p2, bool mx) const {
+        PersistLayout l{};
+        PersistCfg& c = l.c;
+        c.W = W;
+        c.lgW = (W == 1) ? 0 : (W == 2 ? 1 : (W == 4 ? 2 : 3));
+        c.ntiles = (H.nxh + W - 1) / W;
+        c.ppc = ppc;
+        c.rmax = 2 * ppc;
+        c.nres = 11;
+        l.G = std::max(c.ntiles, (H.ny / 2 + ppc - 1) / ppc);
+        const int need = std::max(c.rmax * H.nx / 8, 2 * W * H.ny / 8);
+        l.threads = mx ? pmx_threads(pxa[0], pxa[1], ppc, W) : std::min(256, std::max(64, (need + 31) / 32 * 32));
+        l.smem = p2 ? p2_smem_bytes<T>(H.nx, H.ny, H.ldh, c.rmax, W, c.nres, H.lossy ? 3 : 1)
+                    : (mx ? pmx_smem<T>(pxa[0], pxa[1], c, H.lossy)
+                          : persist_smem_bytes<T>(H.nx, H.ny, H.ldh, c.rmax, W, c.nres));
+        return l;
+    }
 
     pat_status configure_persistent(const HostTables& h) {
         persistent = 0;
@@ -733,10 +796,16 @@ template <typename T> struct Plan : public PlanBase {
         if (!coop) return PAT_OK;
         // power-of-two axes of 16 .. 2048 points take the register-fused kernel
         const char* ep2 = std::getenv("PAT_P2");
-        const bool p2 = !(ep2 && std::atoi(ep2) == 0) && h.fx.pow2 && h.fy.pow2 && h.fx.lgn >= 4 &&
-                        h.fy.lgn >= 4 && h.fx.lgn <= 11 && h.fy.lgn <= 11;
-        const void* kf = p2 ? p2_kernel<T>(false, h.fx.lgn, h.fy.lgn, P.fixed_len) : (const void*)k_persist<T, false>;
-        const void* ka = p2 ? p2_kernel<T>(true, h.fx.lgn, h.fy.lgn, P.fixed_len) : (const void*)k_persist<T, true>;
+        const bool pow2 = !(ep2 && std::atoi(ep2) == 0) && h.fx.pow2 && h.fy.pow2 && h.fx.lgn >= 4 &&
+                          h.fy.lgn >= 4 && h.fx.lgn <= 11 && h.fy.lgn <= 11;
+        // in double the any-length kernel is faster (us a step, absorbing: 66 against 92 at 32^2, 97 against
+        // 116 at 64^2, 91 against 127 at 128^2, 113 against 141 at 256^2)
+        const bool p2 = pow2 && (sizeof(T) == 4 || !mx_2d);
+        const bool mx = !p2 && mx_2d;
+        const void* kf = p2 ? p2_kernel<T>(false, h.fx.lgn, h.fy.lgn, P.fixed_len)
+                            : (mx ? pmx_kernel<T>(false) : (const void*)k_persist<T, false>);
+        const void* ka = p2 ? p2_kernel<T>(true, h.fx.lgn, h.fy.lgn, P.fixed_len)
+                            : (mx ? pmx_kernel<T>(true) : (const void*)k_persist<T, true>);
         cudaError_t e = cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
         if (e != cudaSuccess) {
@@ -749,31 +818,15 @@ template <typename T> struct Plan : public PlanBase {
         int forced_w = 0, forced_p = 0;
         if (const char* ew = std::getenv("PAT_PERSIST_W")) forced_w = std::atoi(ew);
         if (const char* ep = std::getenv("PAT_PERSIST_PPC")) forced_p = std::atoi(ep);
-        struct Cand {
-            PersistCfg c;
-            int G, threads;
-            size_t smem;
-        };
-        std::vector<Cand> ok;
+        std::vector<PersistLayout> ok;
         for (const auto& cnd : cands) {
             const int W = cnd[0], ppc = cnd[1];
             if (forced_w && W != forced_w) continue;
             if (forced_p && ppc != forced_p) continue;
             if (sizeof(T) == 8 && W > 4) continue;
-            const int ntiles = (h.nxh + W - 1) / W;
-            const int npairs = h.ny / 2;
-            const int G = std::max(ntiles, (npairs + ppc - 1) / ppc);
-            PersistCfg c{};
-            c.W = W;
-            c.lgW = (W == 1) ? 0 : (W == 2 ? 1 : (W == 4 ? 2 : 3));
-            c.ntiles = ntiles;
-            c.ppc = ppc;
-            c.rmax = 2 * ppc;
-            c.nres = 11;
-            const int need = std::max(c.rmax * h.nx / 8, 2 * W * h.ny / 8);
-            const int threads = std::min(256, std::max(64, (need + 31) / 32 * 32));
-            const size_t smem = p2 ? p2_smem_bytes<T>(h.nx, h.ny, h.ldh, c.rmax, W, c.nres, h.lossy ? 3 : 1)
-                                   : persist_smem_bytes<T>(h.nx, h.ny, h.ldh, c.rmax, W, c.nres);
+            const PersistLayout l = persist_layout(W, ppc, p2, mx);
+            const int G = l.G, threads = l.threads;
+            const size_t smem = l.smem;
             if (smem > (size_t)optin) continue;
             int per_sm = 0;
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, threads, smem);
@@ -781,22 +834,23 @@ template <typename T> struct Plan : public PlanBase {
             if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, ka, threads, smem);
             if (dbg)
                 fprintf(stderr, "[pat] persistent%s cand W=%d ppc=%d G=%d threads=%d smem=%zu per_sm=%d/%d\n",
-                        p2 ? " (pow2)" : "", W, ppc, G, threads, smem, per_sm, per_sm_a);
+                        p2 ? " (pow2)" : (mx ? " (any length)" : ""), W, ppc, G, threads, smem, per_sm, per_sm_a);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 continue;
             }
             if (std::min(per_sm, per_sm_a) * nsm < G) continue;
-            ok.push_back(Cand{c, G, threads, smem});
+            ok.push_back(l);
         }
         if (ok.empty()) return PAT_OK;
         pat_status st = PAT_OK;
         gbar = dalloc<unsigned>(4, &st);
         if (!gbar) return st;
         persist_p2 = p2;
+        persist_mx = mx;
         persistent = 1;
-        info.path = p2 ? 2 : 1;
-        auto use = [&](const Cand& k) {
+        info.path = pow2 ? 2 : 1;
+        auto use = [&](const PersistLayout& k) {
             pcfg = k.c;
             persist_grid = k.G;
             persist_smem = k.smem;
@@ -825,7 +879,39 @@ template <typename T> struct Plan : public PlanBase {
             if (e2 != cudaSuccess) return cuda_fail(e2, "autotune (persistent kernel)");
             info.tuned = 1;
         }
+        // time reversal runs in k_pmx: the solves' layout where they run in it, else the first that fits
+        if (mx_2d) {
+            if (mx) rev = PersistLayout{pcfg, persist_grid, persist_threads, persist_smem};
+            e = cudaFuncSetAttribute(pmx_kernel<T>(false), cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+            for (const auto& cnd : cands) {
+                if (rev.G || e != cudaSuccess || (sizeof(T) == 8 && cnd[0] > 4)) break;
+                const PersistLayout l = persist_layout(cnd[0], cnd[1], false, true);
+                int per_sm = 0;
+                if (l.smem <= (size_t)optin &&
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pmx_kernel<T>(false), l.threads, l.smem) ==
+                        cudaSuccess &&
+                    per_sm * nsm >= l.G)
+                    rev = l;
+            }
+            if (e != cudaSuccess) cudaGetLastError();
+        }
         return PAT_OK;
+    }
+    // a cooperative launch of k_pmx on plan copy Q (the barrier words are zeroed first)
+    cudaError_t pmx_run(const DevPlan<T>& Q, bool adjoint, const PersistLayout& l, cudaStream_t s) {
+        cudaError_t e = cudaMemsetAsync(gbar, 0, 4 * sizeof(unsigned), s);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(l.G);
+        lc.blockDim = dim3(l.threads);
+        lc.dynamicSmemBytes = l.smem;
+        lc.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+        return pmx_launch<T>(adjoint, &lc, Q, l.c, pxa[0], pxa[1], pxt[0], pxt[1], px_kap, mx_abs, gbar);
     }
 
     pat_status run_persistent(bool adjoint, cudaStream_t s) {
@@ -864,6 +950,8 @@ template <typename T> struct Plan : public PlanBase {
         P.trace_nk = trace_nk;
         if (persist_p2) {
             e = p2_launch<T>(adjoint, &lc, P, pcfg, gbar);
+        } else if (persist_mx) {
+            e = pmx_launch<T>(adjoint, &lc, P, pcfg, pxa[0], pxa[1], pxt[0], pxt[1], px_kap, mx_abs, gbar);
         } else {
             if (adjoint) e = cudaLaunchKernelEx(&lc, k_persist<T, true>, P, pcfg, gbar);
             else e = cudaLaunchKernelEx(&lc, k_persist<T, false>, P, pcfg, gbar);
@@ -1541,6 +1629,13 @@ template <typename T> struct Plan : public PlanBase {
             Q.tr_kc2 = (T)(1.0 / (kc * kc));
         }
         Q.tr_node = tr_node_d;
+        if (D == 2 && rev.G) {   // the whole solve in the persistent kernel
+            Q.data = P.data;
+            Q.trace = nullptr;
+            e = pmx_run(Q, false, rev, s);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(img_out, P.img, N * sizeof(T), cudaMemcpyDefault, s);
+            return e == cudaSuccess ? PAT_OK : cuda_fail(e, "time reversal");
+        }
         // rho^0 = p^0 / (d c0^2), x-FFT of p^0 (its sample goes to the unused row)
         launch(k_fwd_init<T, D>, dim3(G), B, row_smem, s, Q, R, (int)(Nt == 1));
         for (int n = 0; n + 1 < Nt; ++n) {

@@ -34,7 +34,7 @@ def _check(pb, prec):
     assert np.linalg.norm(g - g_ref) <= tol * np.linalg.norm(g_ref)
 
 
-@pytest.mark.parametrize("persist", ["0"])
+@pytest.mark.parametrize("persist", ["0", "1"])
 @pytest.mark.parametrize("prec", ["f32", "f64"])
 @pytest.mark.parametrize("shape", SHAPES_2D, ids=lambda s: "x".join(map(str, s)))
 def test_2d(monkeypatch, shape, prec, persist):
