@@ -416,6 +416,10 @@ template <typename T> struct Plan : public PlanBase {
         use_mx_row = ok[0] && (all || !use_row2) && mx_row_fits(2);
         use_mx_spec = ok[1] && (D == 2 || ok[2]) && (all || !use_spec2) && mx_spec_fits(1);
         mx_2d = D == 2 && ok[0] && ok[1];   // the any-length persistent kernel
+        if (use_mx_row) {   // k_row2 / k_row_u1 are not launched: their shared memory limits no layout
+            use_row2 = use_rowu1 = false;
+            info.rowu1 = 0;
+        }
         pat_status st = PAT_OK;
         for (int a = 0; a < D; ++a) {
             if (mx_2d) {
