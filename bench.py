@@ -169,7 +169,7 @@ def measured_traffic(workload, kernel, version):
 
 def kernel_version(op, fam):
     """Which compiled kernel runs family `fam` on this plan (the captures above are per version)."""
-    if fam.startswith("k_persist"):
+    if fam.startswith(("k_persist", "k_pmx")):
         return fam
     if fam in ("y_fwd", "y_inv"):
         return "k_ywide" if int(getattr(op.info, "ywide", 0)) else "k_spec16"
@@ -820,7 +820,7 @@ def measure(args, name, dev, world, rank, local, with_e2e=True):
                 "share_of_step": share, "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_kind})",
                 "note": ("one persistent launch per solve keeps the state in shared memory (DRAM traffic: "
                          "the set-up loads); the fraction is effective bandwidth of the algorithmic bytes"
-                         if fam.startswith("k_persist") else
+                         if fam.startswith(("k_persist", "k_pmx")) else
                          "per launch: mean algorithmic bytes (operands read and written once) and mean duration "
                          "over this kernel's launches in one forward + adjoint step")}
     # whole-step roofline by the per-point-step algorithmic bytes (state once + medium once)

@@ -934,8 +934,9 @@ template <typename T> struct Plan : public PlanBase {
                 cudaEventCreate(&probe_ev[g][0]);
                 cudaEventCreate(&probe_ev[g][1]);
             }
-            probe_names[g].assign(1, persist_p2 ? (adjoint ? "k_persist2_adj" : "k_persist2_fwd")
-                                                : (adjoint ? "k_persist_adj" : "k_persist_fwd"));
+            probe_names[g].assign(1, persist_p2   ? (adjoint ? "k_persist2_adj" : "k_persist2_fwd")
+                                     : persist_mx ? (adjoint ? "k_pmx_adj" : "k_pmx_fwd")
+                                                  : (adjoint ? "k_persist_adj" : "k_persist_fwd"));
             probe_samples[g] = 1;
             cudaEventRecord(probe_ev[g][0], s);
         }
