@@ -267,64 +267,6 @@ template <typename T, bool INV> __device__ __forceinline__ void mx_row_s0(cplx<T
     });
 }
 
-// last forward stage, R2C unpacking, half spectra of FO fields to global memory
-template <typename T>
-__device__ __forceinline__ void mx_row_out(const cplx<T>* buf, const MxAxis& x, const cplx<T>* tabL,
-                                           cplx<T>* const* spec, int FO, int np, int line0, int ldh) {
-    const int n = x.n, M = x.M, half = n >> 1;
-    const int up = (M - 1) >> 1, us = (M & 1) ? 1 : 2;
-    const int nA = FO * np * up, offA = (nA + 31) & ~31, nB = FO * np * us;
-    with_mx<2>(x.RL, [&](auto RC) PAT_INLINE {
-        constexpr int R = decltype(RC)::value;
-        auto start = [&](cplx<T>(&v)[R], int line, int q) {
-            const cplx<T>* s = buf + line * x.LS + mx_base(x, q);
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = s[r];
-#pragma unroll
-            for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(tabL + (r - 1) * M + q));
-            mx_dft<T, R, false>(v);
-        };
-        for (int t = threadIdx.x; t < offA + nB; t += blockDim.x) {
-            if (t < nA) {
-                const int line = t / up, u = 1 + t - line * up;
-                const int f = line / np, p = line - f * np;
-                cplx<T>* a = spec[f] + (size_t)(line0 + 2 * p) * ldh;
-                cplx<T>* b = a + ldh;
-                cplx<T> v1[R], v2[R];
-                start(v1, line, u);
-                start(v2, line, M - u);
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int k = u + M * r;
-                    const bool low = k <= half;
-                    const int kk = low ? k : n - k;
-                    const cplx<T> zk = v1[r], zm = v2[R - 1 - r];
-                    const T s = low ? (T)0.5 : (T)-0.5;
-                    a[kk] = mkc<T>((T)0.5 * (zk.x + zm.x), s * (zk.y - zm.y));
-                    b[kk] = mkc<T>((T)0.5 * (zk.y + zm.y), s * (zm.x - zk.x));
-                }
-            } else if (t >= offA) {
-                const int w = t - offA;
-                const int line = w / us, q = (w - line * us) ? M >> 1 : 0;
-                const int f = line / np, p = line - f * np;
-                cplx<T>* a = spec[f] + (size_t)(line0 + 2 * p) * ldh;
-                cplx<T>* b = a + ldh;
-                cplx<T> v[R];
-                start(v, line, q);
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int k = q + M * r;
-                    const cplx<T> zk = v[r], zm = q ? v[R - 1 - r] : v[(R - r) % R];
-                    if (k <= half) {
-                        a[k] = mkc<T>((T)0.5 * (zk.x + zm.x), (T)0.5 * (zk.y - zm.y));
-                        b[k] = mkc<T>((T)0.5 * (zk.y + zm.y), (T)0.5 * (zm.x - zk.x));
-                    }
-                }
-            }
-        }
-    });
-}
-
 // One row kernel of a step (Row2Kind); grid nlines / R, or (nlines / R, D) for the u update and its
 // transpose, whose CTAs hold one velocity component.
 template <typename T, int D, int KIND>
