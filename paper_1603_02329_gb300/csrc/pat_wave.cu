@@ -401,7 +401,8 @@ template <typename T> struct Plan : public PlanBase {
     // instances takes 43.2 ms with them and 47.4 ms with k_row2 / k_spec2 for its 256^2 instances) and of
     // double 3-D plans (64^3: 418 against 588 us a step, 80 x 96 x 128: 1182 against 1343).  FP32 3-D and
     // double 2-D plans keep k_row2 / k_spec2 on power-of-two lines (64^3 FP32: 59 against 72 us; 256^2
-    // double: 210 against 283).  PAT_MX=0: none, 2: every line.
+    // double: 210 against 283).  PAT_MX=0: none, 2: every line; PAT_ROW2=0, PAT_SPEC2=0: the generic row,
+    // spectral kernels.
     pat_status build_mx(const HostTables& h) {
         const char* ev = std::getenv("PAT_MX");
         const int mode = ev ? std::atoi(ev) : 1;
@@ -413,8 +414,12 @@ template <typename T> struct Plan : public PlanBase {
         bool ok[3] = {};
         for (int a = 0; a < D; ++a) ok[a] = mx_axis(n[a], mx_r1max<T>(), 0, &mxa[a]);
         const bool all = mode == 2 || (D == 2) == (sizeof(T) == 4);
-        use_mx_row = ok[0] && (all || !use_row2) && mx_row_fits(2);
-        use_mx_spec = ok[1] && (D == 2 || ok[2]) && (all || !use_spec2) && mx_spec_fits(1);
+        const auto off = [](const char* name) {
+            const char* e = std::getenv(name);
+            return e && std::atoi(e) == 0;
+        };
+        use_mx_row = ok[0] && !off("PAT_ROW2") && (all || !use_row2) && mx_row_fits(2);
+        use_mx_spec = ok[1] && (D == 2 || ok[2]) && !off("PAT_SPEC2") && (all || !use_spec2) && mx_spec_fits(1);
         mx_2d = D == 2 && ok[0] && ok[1];   // the any-length persistent kernel
         if (use_mx_row) {   // k_row2 / k_row_u1 are not launched: their shared memory limits no layout
             use_row2 = use_rowu1 = false;
@@ -798,14 +803,15 @@ template <typename T> struct Plan : public PlanBase {
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
         const bool dbg = std::getenv("PAT_DEBUG") != nullptr;
         if (!coop) return PAT_OK;
-        // power-of-two axes of 16 .. 2048 points take the register-fused kernel
+        // power-of-two axes of 16 .. 2048 points take the register-fused kernel; PAT_P2=0: the generic one
         const char* ep2 = std::getenv("PAT_P2");
-        const bool pow2 = !(ep2 && std::atoi(ep2) == 0) && h.fx.pow2 && h.fy.pow2 && h.fx.lgn >= 4 &&
+        const bool generic = ep2 && std::atoi(ep2) == 0;
+        const bool pow2 = !generic && h.fx.pow2 && h.fy.pow2 && h.fx.lgn >= 4 &&
                           h.fy.lgn >= 4 && h.fx.lgn <= 11 && h.fy.lgn <= 11;
         // in double the any-length kernel is faster (us a step, absorbing: 66 against 92 at 32^2, 97 against
         // 116 at 64^2, 91 against 127 at 128^2, 113 against 141 at 256^2)
         const bool p2 = pow2 && (sizeof(T) == 4 || !mx_2d);
-        const bool mx = !p2 && mx_2d;
+        const bool mx = !generic && !p2 && mx_2d;
         const void* kf = p2 ? p2_kernel<T>(false, h.fx.lgn, h.fy.lgn, P.fixed_len)
                             : (mx ? pmx_kernel<T>(false) : (const void*)k_persist<T, false>);
         const void* ka = p2 ? p2_kernel<T>(true, h.fx.lgn, h.fy.lgn, P.fixed_len)

@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     ((60, 56), "f64", {}, "k_pmx"),
     ((60, 56), "f32", {"PAT_MX": "0"}, "k_persist"),
     ((64, 64), "f64", {"PAT_MX": "0"}, "k_persist2"),
+    ((64, 64), "f32", {"PAT_P2": "0"}, "k_persist"),
+    ((64, 64), "f64", {"PAT_P2": "0"}, "k_persist"),
+    ((60, 56), "f64", {"PAT_P2": "0"}, "k_persist"),
 ])
 def test_persistent_kernel_is_named(monkeypatch, shape, prec, env, name):
     from paper_1603_02329_gb300.api import PATOperator
@@ -33,3 +36,26 @@ def test_persistent_kernel_is_named(monkeypatch, shape, prec, env, name):
     assert [s[0] for s in op.probe(False)] == [name + "_fwd"]
     assert [s[0] for s in op.probe(True)] == [name + "_adj"]
     op.close()
+
+
+# PAT_ROW2=0 and PAT_SPEC2=0 select the generic row and spectral kernels, whatever the mixed-radix kernels
+# would take: the same bits as with those kernels off
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("shape", [(32, 64), (30, 48), (16, 16, 32), (12, 20, 18)], ids=lambda s: "x".join(map(str, s)))
+def test_generic_per_phase_kernels_are_selected(monkeypatch, shape, prec):
+    from paper_1603_02329_gb300.api import PATOperator
+
+    make = synth.small_lossy_2d if len(shape) == 2 else synth.small_lossy_3d
+    pb = make(shape=shape, pml=2, Nt=12)
+    for k in ("PAT_PERSIST", "PAT_AUTOTUNE", "PAT_ROW2", "PAT_SPEC2"):
+        monkeypatch.setenv(k, "0")
+    out = []
+    for mx in ("1", "0"):
+        monkeypatch.setenv("PAT_MX", mx)
+        op = PATOperator.from_problem(pb, precision=prec, device=torch.device("cuda", 0))
+        assert op.info.path == 0
+        h = torch.tensor(np.random.default_rng(3).standard_normal((pb.Nt, op.Ns)), device="cuda",
+                         dtype=torch.float32 if prec == "f32" else torch.float64)
+        out.append(([int(v) for v in op.info.layout], op.adjoint(h).cpu().numpy()))
+        op.close()
+    assert out[0][0] == out[1][0] and np.array_equal(out[0][1], out[1][1])
