@@ -33,13 +33,15 @@ constexpr bool mx_radix(int r) { return (r >= 2 && r <= 10) || r == 12 || r == 1
 inline unsigned mx_magic(int d) { return d == 1 ? 0u : (unsigned)(((1ull << 32) + d - 1) / d); }
 
 // The schedule of an even length; false when there is none.  r1max: 16, or 10 in double (registers).
-//   stage = 0 (the per-phase kernels): two stages where the radices allow it, else three, with the smallest
-//   largest radix.  Radices stay small on purpose: the outer stages are unrolled code that every warp runs
-//   once per launch, and with radices up to 16 (two stages for most lines up to 256) the kernels waited for
-//   instructions (4 to 9 stall cycles per issue, 128 registers).
-//   stage > 0 (the persistent kernel): the least work of one thread over all stages, where the last stage
-//   counts twice (its threads run two butterflies) and a third stage costs `stage`.  With a butterfly or
-//   less per thread a phase takes as long as its longest threads.
+//   stage = 0 (the FP32 per-phase kernels): two stages where the radices allow it, else three, with the
+//   smallest largest radix.  Radices stay small on purpose: the outer stages are unrolled code that every warp
+//   runs once per launch, and with radices up to 16 (two stages for most lines up to 256) the kernels waited
+//   for instructions (4 to 9 stall cycles per issue, 128 registers).
+//   stage > 0 (the persistent kernel, and the per-phase kernels in double): the least work of one thread over
+//   all stages, where the last stage counts twice (its threads run two butterflies) and a third stage costs
+//   `stage`.  With a butterfly or less per thread a phase takes as long as its longest threads, the more so in
+//   double, where an instruction holds its pipe for 64 clocks (30 x 50 x 70 FP64, us a step: 318 against 450
+//   with the two-stage schedules of radices up to 10 and 350 in the generic kernels; 54^2: 71, 118, 80).
 inline bool mx_axis(int n, int r1max, int stage, MxAxis* out) {
     int best = 1 << 30;
     MxAxis a{};

@@ -396,13 +396,20 @@ template <typename T> struct Plan : public PlanBase {
     int mx_w = 1;          // columns per spectral CTA
     int optin_smem = 0;
 
-    // Lines that are no power of two take these kernels where a schedule exists, and so do all lines of FP32
-    // 2-D plans (their per-phase kernels run in batches and gradients, untuned: the batch of eight uneven
-    // instances takes 43.2 ms with them and 47.4 ms with k_row2 / k_spec2 for its 256^2 instances) and of
-    // double 3-D plans (64^3: 418 against 588 us a step, 80 x 96 x 128: 1182 against 1343).  FP32 3-D and
-    // double 2-D plans keep k_row2 / k_spec2 on power-of-two lines (64^3 FP32: 59 against 72 us; 256^2
-    // double: 210 against 283).  PAT_MX=0: none, 2: every line; PAT_ROW2=0, PAT_SPEC2=0: the generic row,
-    // spectral kernels.
+    // Which lines take these kernels (us a step, one instance, against the kernels they replace).  Where they
+    // have a schedule:
+    //   no power of two: all but the row kernels of double 2-D plans with fewer than 512 lines of more than 64
+    //     points.  There a CTA's few long butterflies leave double pipes idle that the generic row kernels' many
+    //     short ones use (300^2: 312 with both, 227 with the y passes alone, generic 290; 150 x 400: 310, 164,
+    //     205; but 60^2: 73, 76, 87, and 720^2: 650, 770, 910);
+    //   powers of two, FP32 2-D: all (128^2: 36 against 47 with k_row2 / k_spec2; the batch of eight uneven
+    //     instances takes 44.2 ms and with k_row2 on its 256-point lines 47.4).  512^2 takes 68 against 69 and
+    //     1024^2 105 against 91: there for the smaller error (gradient of 1024^2, 200 steps: 1.7e-6 against
+    //     3.1e-6; of 1024 x 64, 300 steps: 1.6e-6 against 5.6e-6; see k_mx_kap).  FP32 3-D: none (64^3: 72
+    //     against 59);
+    //   powers of two, double: 3-D only (64^3: 353 against 560, 128^3: 2290 against 3270, 256^3: 19600
+    //     against 25500; 2-D 256^2: 283 against 210).
+    // PAT_MX=0: none, 2: every line; PAT_ROW2=0, PAT_SPEC2=0: the generic row, spectral kernels.
     pat_status build_mx(const HostTables& h) {
         const char* ev = std::getenv("PAT_MX");
         const int mode = ev ? std::atoi(ev) : 1;
@@ -412,14 +419,16 @@ template <typename T> struct Plan : public PlanBase {
         cudaDeviceGetAttribute(&optin_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         const int D = h.d, n[3] = {h.nx, h.ny, h.nz};
         bool ok[3] = {};
-        for (int a = 0; a < D; ++a) ok[a] = mx_axis(n[a], mx_r1max<T>(), 0, &mxa[a]);
-        const bool all = mode == 2 || (D == 2) == (sizeof(T) == 4);
+        const bool f32 = sizeof(T) == 4;
+        for (int a = 0; a < D; ++a) ok[a] = mx_axis(n[a], mx_r1max<T>(), f32 ? 0 : 4, &mxa[a]);
         const auto off = [](const char* name) {
             const char* e = std::getenv(name);
             return e && std::atoi(e) == 0;
         };
-        use_mx_row = ok[0] && !off("PAT_ROW2") && (all || !use_row2) && mx_row_fits(2);
-        use_mx_spec = ok[1] && (D == 2 || ok[2]) && !off("PAT_SPEC2") && (all || !use_spec2) && mx_spec_fits(1);
+        const bool row = f32 ? D == 2 || !use_row2 : D == 3 || (!use_row2 && (h.nx <= 64 || h.ny >= 512));
+        const bool spec = !use_spec2 || (D == 2) == f32;
+        use_mx_row = ok[0] && !off("PAT_ROW2") && (mode == 2 || row) && mx_row_fits(2);
+        use_mx_spec = ok[1] && (D == 2 || ok[2]) && !off("PAT_SPEC2") && (mode == 2 || spec) && mx_spec_fits(1);
         mx_2d = D == 2 && ok[0] && ok[1];   // the any-length persistent kernel
         if (use_mx_row) {   // k_row2 / k_row_u1 are not launched: their shared memory limits no layout
             use_row2 = use_rowu1 = false;
@@ -457,7 +466,7 @@ template <typename T> struct Plan : public PlanBase {
                 if (P.nlines % r == 0 && mx_row_fits(r)) break;
             }
         if (use_mx_spec) {
-            mx_w = std::getenv("PAT_COL_W") ? cfg.col_w : 4;
+            mx_w = std::getenv("PAT_COL_W") ? cfg.col_w : (f32 || D == 3 ? 4 : 2);
             while (mx_w > 1 && !mx_spec_fits(mx_w)) mx_w /= 2;
         }
         return PAT_OK;

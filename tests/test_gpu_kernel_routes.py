@@ -59,3 +59,22 @@ def test_generic_per_phase_kernels_are_selected(monkeypatch, shape, prec):
         out.append(([int(v) for v in op.info.layout], op.adjoint(h).cpu().numpy()))
         op.close()
     assert out[0][0] == out[1][0] and np.array_equal(out[0][1], out[1][1])
+
+
+# Which family the untuned per-phase kernels are from, as the launch layout shows it: (columns per spectral
+# CTA, x-lines per row CTA) are (4 or in double 2-D 2, 8 / 4 / 2) with the mixed-radix kernels, (2 or in
+# double 1, 2) with the others
+@pytest.mark.parametrize("shape,prec,layout", [
+    ((48, 512), "f32", (4, 8)), ((48, 60), "f64", (2, 8)), ((48, 300), "f64", (2, 2)), ((64, 300), "f64", (1, 2)),
+    ((540, 100), "f64", (2, 4)),
+    ((12, 20, 300), "f64", (4, 8)), ((16, 16, 64), "f64", (4, 8)), ((16, 16, 64), "f32", (2, 2)),
+], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else v)
+def test_untuned_kernel_family(monkeypatch, shape, prec, layout):
+    from paper_1603_02329_gb300.api import PATOperator
+
+    monkeypatch.setenv("PAT_PERSIST", "0")
+    monkeypatch.setenv("PAT_AUTOTUNE", "0")
+    make = synth.small_lossy_2d if len(shape) == 2 else synth.small_lossy_3d
+    op = PATOperator.from_problem(make(shape=shape, pml=2, Nt=4), precision=prec, device=torch.device("cuda", 0))
+    assert (op.info.layout[0], op.info.layout[1]) == layout
+    op.close()
