@@ -566,9 +566,14 @@ template <typename T> __global__ void k_mx_kap(MxTableArgs A, T* kap, T* abs) {
         const double kxv = A.kv[0][min(kx, A.nxh - 1)], klv = A.kv[la][kl];
         double k2 = kxv * kxv + klv * klv;
         if (A.d == 3) k2 += A.kv[1][ko] * A.kv[1][ko];
-        kap[i] = (T)(sinc_sq(A.kap_a * A.kap_a * k2) * A.invN * A.scale);
+        if (kap) kap[i] = (T)(sinc_sq(A.kap_a * A.kap_a * k2) * A.invN * A.scale);
         if (abs) {
-            abs[i] = (k2 > 0.0) ? (T)(pow(k2, A.pha) * A.invN) : (T)0;
+            double win = 1.0;
+            if (A.tr_kc2 > 0.0) {   // time reversal: reversed and windowed
+                const double q2 = k2 * A.tr_kc2, q = sqrt(q2);
+                win = q2 < 1.0 ? -(0.42 + 0.5 * cospi(q) + 0.08 * cospi(2.0 * q)) : 0.0;
+            }
+            abs[i] = (k2 > 0.0) ? (T)(win * pow(k2, A.pha) * A.invN) : (T)0;
             abs[n + i] = (k2 > 0.0) ? (T)(pow(k2, A.phb) * A.invN) : (T)0;
         }
     }
@@ -597,13 +602,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_mx_spec(DevPlan
     const int kx = min(kx0 + c, P.nxh - 1);
     cplx<T> mx = mkc<T>(0, 0), mo = mkc<T>(0, 0);
     const cplx<T>* ml = nullptr;
-    T ck2 = 0;
-    const bool tabled = MODE != SPEC_ABS || mt != nullptr;
     if constexpr (MUL) {
         mx = plus ? P.dp[0][kx] : P.dm[0][kx];
         ml = plus ? P.dp[lax] : P.dm[lax];
         if (D == 3) mo = plus ? P.dp[1][outer] : P.dm[1][outer];
-        ck2 = P.kv[0][kx] * P.kv[0][kx];
     }
     pdl_trigger();
     pdl_wait();
@@ -763,15 +765,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_mx_spec(DevPlan
                         for (int r = 0; r < R; ++r) {
                             const int k = q + M * r;
                             if constexpr (MODE == SPEC_ABS) {
-                                T sc;
-                                if (tabled) sc = mult(k);
-                                else {
-                                    const T kl = P.kv[lax][k];
-                                    T k2 = ck2 + kl * kl;
-                                    if (D == 3) k2 += P.kv[1][outer] * P.kv[1][outer];
-                                    sc = (f0 == 0) ? abs_mult0(P, k2) : ((k2 > (T)0) ? pow(k2, P.phb) * P.invN : (T)0);
-                                }
-                                v[r] = cscale(v[r], sc);
+                                v[r] = cscale(v[r], mult(k));
                             } else {
                                 const T sc = mult(k);
                                 v[r] = cscale(cmul(v[r], shift(f0, k)), (MODE == SPEC_DIVT) ? -sc : sc);

@@ -176,18 +176,18 @@ inline int mx_spec_threads(const MxAxis& a, int W) {
     const int b = std::max(a.m0, std::max(a.M, a.R1 > 1 ? a.R0 * a.RL : 0));
     return std::max(32, std::min(256, (b * W + 31) / 32 * 32));
 }
-// mt: kappa / N ([outer][line][ldh]) for the derivative modes, the two absorption tables or nullptr
-// (computed inline) for SPEC_ABS
+// mt: kappa / N ([outer][line][ldh]) for the derivative modes, the two absorption tables for SPEC_ABS
 template <typename T>
 cudaError_t mx_spec_launch(const cudaLaunchConfig_t* lc, int D, int mode, const DevPlan<T>& P, const MxAxis& a,
                            const cplx<T>* tw, int W, int lax, const T* mt);
 template <typename T> cudaError_t mx_spec_attrs(int bytes);
-// fill the multiplier tables of the plan (kappa / N; |k|^(y-2) / N and |k|^(y-1) / N when abs != nullptr)
+// fill multiplier tables of the plan (kappa / N; |k|^(y-2) / N and |k|^(y-1) / N; either may be nullptr)
 struct MxTableArgs {
     int d, ny, nz, nxh, ldh;
     const double* kv[3];   // wavenumbers per axis (device)
     double kap_a, pha, phb, invN;
     double scale;          // of kappa: takes out mean rounding errors (k_mx_kap)
+    double tr_kc2;         // > 0: |k|^(y-2) / N reversed and windowed at 1 / sqrt(tr_kc2) (time reversal)
 };
 template <typename T> cudaError_t mx_tables(const MxTableArgs& A, T* kap, T* abs, cudaStream_t s);
 

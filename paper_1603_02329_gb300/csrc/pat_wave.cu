@@ -393,6 +393,7 @@ template <typename T> struct Plan : public PlanBase {
     double mx_gain_sum = 0.0, px_gain = 0.0;
     const double* mx_kv[3] = {nullptr, nullptr, nullptr};
     T* mx_abs = nullptr;   // |k|^(y-2) / N and |k|^(y-1) / N, [2][outer][line][ldh] (absorbing plans)
+    T* mx_tr = nullptr;    // the same with time reversal's window, filled by each such call
     int mx_w = 1;          // columns per spectral CTA
     int optin_smem = 0;
 
@@ -483,9 +484,12 @@ template <typename T> struct Plan : public PlanBase {
                 return false;
         return true;
     }
+    MxTableArgs mx_table_args() const {
+        return {H.d, H.ny, H.nz, H.nxh, H.ldh, {mx_kv[0], mx_kv[1], mx_kv[2]}, H.kap_a, H.pha, H.phb, H.invN, 1.0, 0.0};
+    }
     pat_status build_mx_tables() {
         if (!mx_kap) return PAT_OK;
-        MxTableArgs A{H.d, H.ny, H.nz, H.nxh, H.ldh, {mx_kv[0], mx_kv[1], mx_kv[2]}, H.kap_a, H.pha, H.phb, H.invN, 1.0};
+        MxTableArgs A = mx_table_args();
         double dts = 1.0, gm = 0.0, gp = 0.0;
         if (sizeof(T) == 4) {   // in double such errors are below the transforms' own
             // dt, and the medium's mean rounding error (of a homogeneous one, the same at every point): kappa
@@ -528,12 +532,12 @@ template <typename T> struct Plan : public PlanBase {
         note_launch(D == 2 ? mx_row_launch_d<T, 2>(&lc, kind, Q, mxa[0], mxt[0], R, flag, data_row, h_row, qrow, gc2, p0c)
                            : mx_row_launch_d<T, 3>(&lc, kind, Q, mxa[0], mxt[0], R, flag, data_row, h_row, qrow, gc2, p0c));
     }
-    // F: fields of a plain transform; the absorption tables hold no time-reversal window
+    // F: fields of a plain transform
     void mx_spec(int mode, const DevPlan<T>& Q, cudaStream_t s, int lax, int F) {
         const int D = Q.d, W = mx_w;
         const bool one = mode == SPEC_GRAD || mode == SPEC_GRADT;
         const int fields = one ? 1 : (mode == SPEC_ABS ? 2 : (mode == SPEC_PLAIN_FWD || mode == SPEC_PLAIN_INV ? F : D));
-        const T* mt = mode != SPEC_ABS ? mx_kap : (Q.tr_kc2 > (T)0 ? nullptr : mx_abs);
+        const T* mt = mode != SPEC_ABS ? mx_kap : (Q.tr_kc2 > (T)0 ? mx_tr : mx_abs);
         cudaLaunchConfig_t lc = {};
         lc.gridDim = dim3(fields, (Q.nxh + W - 1) / W, lax == 1 ? Q.nz : Q.ny);
         lc.blockDim = dim3(mx_spec_threads(mxa[lax], W));
@@ -1600,6 +1604,10 @@ template <typename T> struct Plan : public PlanBase {
             aux_rows = dalloc<T>((size_t)(std::max(H.Nt - 1, 1) + 1) * std::max(H.Ns, 1), &st);
             if (!aux_rows) return st;
         }
+        if (tr && !mx_tr && use_mx_spec && P.lossy && !rev.G) {
+            mx_tr = dalloc<T>(2 * (size_t)H.ny * H.nz * H.ldh, &st);
+            if (!mx_tr) return st;
+        }
         if (tr && !tr_node_d) {
             std::vector<int> node;
             st = tr_nodes(node);
@@ -1639,8 +1647,8 @@ template <typename T> struct Plan : public PlanBase {
         DevPlan<T> Q = P;
         Q.data = junk;
         Q.spec16 = std::min(Q.spec16, 1);
+        double kc = 0.0;
         if (compensate) {
-            double kc = 0.0;
             for (int a = 0; a < D; ++a) {
                 const double kn = M_PI / in.grid.dx[a];
                 kc = (a == 0) ? kn : std::min(kc, kn);
@@ -1655,6 +1663,13 @@ template <typename T> struct Plan : public PlanBase {
             e = pmx_run(Q, false, rev, s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(img_out, P.img, N * sizeof(T), cudaMemcpyDefault, s);
             return e == cudaSuccess ? PAT_OK : cuda_fail(e, "time reversal");
+        }
+        if (mx_tr && compensate) {
+            // one pow and two cospi per mode and call; formed in the passes instead they made a time-reversal
+            // step in double a quarter longer than a forward one
+            MxTableArgs A = mx_table_args();
+            A.tr_kc2 = 1.0 / (kc * kc);
+            note_launch(mx_tables<T>(A, nullptr, mx_tr, s));
         }
         // rho^0 = p^0 / (d c0^2), x-FFT of p^0 (its sample goes to the unused row)
         launch(k_fwd_init<T, D>, dim3(G), B, row_smem, s, Q, R, (int)(Nt == 1));
