@@ -493,8 +493,9 @@ template <typename T> struct Plan : public PlanBase {
         double dts = 1.0, gm = 0.0, gp = 0.0;
         if (sizeof(T) == 4) {   // in double such errors are below the transforms' own
             // dt, and the medium's mean rounding error (of a homogeneous one, the same at every point): kappa
-            // scales D+ and D-, so it takes half of that of b rho0 c0^2
-            const size_t N = (size_t)P.N, step = std::max<size_t>(1, N >> 20);
+            // scales D+ and D-, so it takes half of that of b rho0 c0^2.  A sample of 2^14 points at an odd
+            // stride (its mean is good to 2e-10; every point of 512^2 took 2 ms of a plan's 16)
+            const size_t N = (size_t)P.N, step = std::max<size_t>(1, N >> 14) | 1;
             double med = 0.0;
             size_t cnt = 0;
             const auto err = [](double v) { return (double)(T)v / v - 1.0; };
@@ -881,9 +882,10 @@ template <typename T> struct Plan : public PlanBase {
         };
         use(ok[0]);   // least work per CTA first
         if (ok.size() > 1 && autotune_enabled() && !forced_w && !forced_p && H.Nt >= 2) {
-            // autotuner: time a short forward solve (at most 24 steps) with each co-resident layout
+            // autotuner: time a short forward solve (at most 24 steps, 8 in double, whose steps are three
+            // times as long and whose layouts are up to ten) with each co-resident layout
             const int Nt_full = P.Nt;
-            P.Nt = std::min(Nt_full, 24);
+            P.Nt = std::min(Nt_full, sizeof(T) == 4 ? 24 : 8);
             size_t bi = 0;
             float best = 1e30f;
             for (size_t i = 0; i < ok.size(); ++i) {
