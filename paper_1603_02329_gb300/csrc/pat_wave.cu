@@ -467,7 +467,9 @@ template <typename T> struct Plan : public PlanBase {
                 if (P.nlines % r == 0 && mx_row_fits(r)) break;
             }
         if (use_mx_spec) {
-            mx_w = std::getenv("PAT_COL_W") ? cfg.col_w : (f32 || D == 3 ? 4 : 2);
+            mx_w = f32 || D == 3 ? 4 : 2;
+            if (const char* ew = std::getenv("PAT_COL_W"))   // up to the tuner's widest
+                for (mx_w = 1; 2 * mx_w <= std::min(std::atoi(ew), f32 ? 16 : 8);) mx_w *= 2;
             while (mx_w > 1 && !mx_spec_fits(mx_w)) mx_w /= 2;
         }
         return PAT_OK;
@@ -701,13 +703,14 @@ template <typename T> struct Plan : public PlanBase {
             scheds = {P.spec16};
             chunk_cands = {1};
         }
+        const int pin_w = use_mx_spec ? mx_w : base.col_w;
         int best_mxw = mx_w;
         std::vector<int> widths{1, 2, 4, 8};
         if (use_mx_spec && sizeof(T) == 4) widths.push_back(16);
         for (int nchunk : chunk_cands)
         for (int sched : scheds)
         for (int w : widths) {
-            if (fw && w != base.col_w) continue;
+            if (fw && w != pin_w) continue;
             if (sizeof(T) == 8 && w > (use_mx_spec ? 8 : 4)) continue;
             for (int r : {2, 4, 8, 16}) {
                 if (fr && r != base.row_lines) continue;
