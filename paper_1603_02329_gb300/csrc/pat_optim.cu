@@ -50,17 +50,24 @@ template <typename T> __device__ __forceinline__ T dfwd(const T* x, long long i,
 // One FGP iteration (dual of the TV prox, Sec. IV): r = q + w (q - q_prev), then
 // q_new = Pi_{|q|<=1}(r + step D x(r)) with x(r) = P_C(z - lam D^T r).
 //
-// Bound by memory: z and the last two duals read, the new one written, 1 + 3 d fields per iteration
-// (r is formed where it is read, so it is never stored).  A CTA takes a TX x TY tile of (x, y) and
-// marches along z over `chunk` planes; each plane's x(r) goes once through shared memory with a halo of
-// one column and one row, and r_z of the plane below and the plane above's x(r) stay in registers, so
-// a field is fetched from DRAM about once.  256^3 FP32: the map of 20 iterations takes 4.25 ms (0.21 ms
-// an iteration, 3.2 TB/s of the 1 + 3 d fields) against 20.2 ms for one thread per point over flat
-// indices, which formed x(r) d + 1 times from global memory, stored r, and divided 64-bit indices.
+// A CTA takes a tile of (x, y) and marches along z over `chunk` planes.  Each plane's x(r) goes once through
+// shared memory with a halo of one column and one row; the next plane's is formed before the barrier, so its
+// loads are in flight there, and r is formed where it is read and kept in registers for the plane's update.
+// FP32 is bound by memory: z and the last two duals read, the new one written, 1 + 3 d fields per iteration,
+// each fetched from DRAM about once (256^3, 20 iterations: 3.65 ms, 3.7 TB/s; 4.25 ms with the next plane after
+// the barrier; 20 ms for one thread per point over flat indices, which formed x(r) d + 1 times from global
+// memory).  Its 64 x 8 tile is compiled in: run-time sides cost a quarter (256^3: 5.9 against 4.8 ms).  Images of at most 32 columns would leave half of its lanes idle, and
+// double is bound by its pipes, where an idle lane costs as much as a busy one: both take a run-time tile whose
+// points fill the CTA's lanes (fgp_tile).  20 iterations, flat / 64 x 8 tiles / run-time tiles, in us:
+// 1000 x 1000 x 4 FP32 4220 / 8260 / 1360; 256 x 256 x 8 FP32 740 / 790 / 290; double 1000 x 1000 x 4 10800 /
+// 58400 / 8200, 64^3 1040 / 1330 / 800, 256^2 376 / 439 / 323, 256^3 44400 / 32800 / 31900.
 constexpr int kFgpX = 64, kFgpY = 8;
+constexpr int kFgpThreads = 512;   // tile points, and threads, of a CTA
+constexpr int kFgpRows = 256;      // rows of a tile
 
 template <typename T> struct FgpArgs {
     int nx, ny, nz, chunk;   // chunk: planes per CTA (3-D)
+    int tw, th;              // points of a tile along x and y
     unsigned gx, gy;         // tiles along x and y (the grid is one-dimensional: no limit on a side)
     const T* z;
     const T* q[3];           // q_k
@@ -70,12 +77,14 @@ template <typename T> struct FgpArgs {
     int nonneg, first;       // first: q_k = q_{k-1} = 0 (not read)
 };
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kFgpX * kFgpY) k_fgp_iter(FgpArgs<T> A) {
-    __shared__ T sx[2][kFgpY + 1][kFgpX + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kFgpX + tx;
+template <typename T, int D, bool FIXED>
+__global__ void __launch_bounds__(kFgpThreads) k_fgp_iter(FgpArgs<T> A) {
+    // (tw + 1)(th + 1), at most kFgpThreads + kFgpRows + 3
+    __shared__ T sx[2][FIXED ? (kFgpX + 1) * (kFgpY + 1) : kFgpThreads + kFgpRows + 4];
+    const int tw = FIXED ? kFgpX : A.tw, th = FIXED ? kFgpY : A.th, ld = tw + 1;
+    const int tid = threadIdx.x, ty = tid / tw, tx = tid - ty * tw;
     const unsigned bx = blockIdx.x % A.gx, byz = blockIdx.x / A.gx, by = byz % A.gy, bz = byz / A.gy;
-    const int x0 = bx * kFgpX, y0 = by * kFgpY;
+    const int x0 = bx * tw, y0 = by * th;
     const int k0 = (D == 3) ? bz * A.chunk : 0;
     const int k1 = (D == 3) ? min(k0 + A.chunk, A.nz) : 1;
     const int nx = A.nx, ny = A.ny;
@@ -112,60 +121,61 @@ __global__ void __launch_bounds__(kFgpX * kFgpY) k_fgp_iter(FgpArgs<T> A) {
     };
 
     const int x = x0 + tx, y = y0 + ty;
-    const bool in = x < nx && y < ny;
-    // this thread's halo point, if any: the column x0 + TX (rows 0 .. TY - 1), the row y0 + TY
+    const bool in = ty < th && x < nx && y < ny;
+    // this thread's halo point, if any: the column x0 + tw (rows 0 .. th - 1), the row y0 + th
     int hx = -1, hy = 0;
-    if (tid < kFgpY) {
-        hx = kFgpX;
+    if (FIXED) {
+        if (tid < th) {
+            hx = tw;
+            hy = tid;
+        } else if (tid >= 32 && tid < 32 + tw) {
+            hx = tid - 32;
+            hy = th;
+        }
+    } else if (tid < th) {
+        hx = tw;
         hy = tid;
-    } else if (tid >= 32 && tid < 32 + kFgpX) {
-        hx = tid - 32;
-        hy = kFgpY;
+    } else if (tid < th + tw) {
+        hx = tid - th;
+        hy = th;
     }
     const bool hin = hx >= 0 && x0 + hx < nx && y0 + hy < ny;
     const size_t i0 = (size_t)y * sy + x, h0 = (size_t)(y0 + hy) * sy + (x0 + (hx < 0 ? 0 : hx));
-    T rp[3] = {0, 0, 0}, gx = 0, gy = 0, xp = 0, rzm = 0, hrzm = 0;
+    const int at = ty * ld + tx;
+    T r[3] = {0, 0, 0}, xk = 0, rzm = 0, hrzm = 0;
     if (D == 3 && k0 >= 1 && !A.first) {
         if (in) rzm = r_at(2, i0 + (size_t)(k0 - 1) * sz);
         if (hin) hrzm = r_at(2, h0 + (size_t)(k0 - 1) * sz);
     }
-    // plane k1 (3-D) only gives x(r) to plane k1 - 1's difference along z
-    const int kend = (D == 3 && k1 < A.nz) ? k1 : k1 - 1;
-    for (int k = k0; k <= kend; ++k) {
-        T r[3] = {0, 0, 0}, hr[3] = {0, 0, 0};
-        T xk = 0;
-        T(&s)[kFgpY + 1][kFgpX + 1] = sx[(k - k0) & 1];
-        if (in) xk = prox(x, y, k, i0 + (size_t)k * sz, rzm, r);
-        if (k < k1) {
-            s[ty][tx] = xk;
-            if (hin) {
-                s[hy][hx] = prox(x0 + hx, y0 + hy, k, h0 + (size_t)k * sz, hrzm, hr);
-                hrzm = hr[2];
-            }
+    if (in) xk = prox(x, y, k0, i0 + (size_t)k0 * sz, rzm, r);
+    for (int k = k0; k < k1; ++k) {
+        T* s = sx[(k - k0) & 1];
+        if (in) s[at] = xk;
+        if (hin) {
+            T hr[3];
+            s[hy * ld + hx] = prox(x0 + hx, y0 + hy, k, h0 + (size_t)k * sz, hrzm, hr);
+            if constexpr (D == 3) hrzm = hr[2];
         }
+        // the next plane's x(r), for this plane's difference along z; its loads are in flight at the barrier
+        const bool up = D == 3 && k + 1 < A.nz;
+        T rn[3] = {0, 0, 0}, xn = 0;
+        if (in && up) xn = prox(x, y, k + 1, i0 + (size_t)(k + 1) * sz, r[2], rn);
         __syncthreads();
-        auto put = [&](int kk, const T* rr, T g0, T g1, T g2) {   // q_new of plane kk
-            T q[3] = {rr[0] + A.step * g0, rr[1] + A.step * g1, (D == 3) ? rr[2] + A.step * g2 : (T)0};
+        if (in) {
+            T q[3] = {r[0] + A.step * ((x < nx - 1) ? s[at + 1] - xk : (T)0),
+                      r[1] + A.step * ((y < ny - 1) ? s[at + ld] - xk : (T)0),
+                      (D == 3) ? r[2] + A.step * (up ? xn - xk : (T)0) : (T)0};
             T nrm2 = 0;
 #pragma unroll
             for (int a = 0; a < D; ++a) nrm2 += q[a] * q[a];
-            const T sc = (T)1 / fmax((T)1, sqrt(nrm2));
+            T sc = (T)1;   // of |q| <= 1 and of NaN: in double the branch saves a division and a root
+            if (sizeof(T) == 4 || nrm2 > (T)1) sc = (T)1 / fmax((T)1, sqrt(nrm2));
 #pragma unroll
-            for (int a = 0; a < D; ++a) A.qn[a][i0 + (size_t)kk * sz] = q[a] * sc;
-        };
-        if (in) {
-            if (D == 3 && k > k0) put(k - 1, rp, gx, gy, xk - xp);
-            if (k < k1) {
-                gx = (x < nx - 1) ? s[ty][tx + 1] - xk : (T)0;
-                gy = (y < ny - 1) ? s[ty + 1][tx] - xk : (T)0;
-                if (D == 2) put(k, r, gx, gy, (T)0);
-                else if (k == A.nz - 1) put(k, r, gx, gy, (T)0);
-            }
+            for (int a = 0; a < D; ++a) A.qn[a][i0 + (size_t)k * sz] = q[a] * sc;
         }
 #pragma unroll
-        for (int a = 0; a < 3; ++a) rp[a] = r[a];
-        xp = xk;
-        rzm = r[2];
+        for (int a = 0; a < 3; ++a) r[a] = rn[a];
+        xk = xn;
     }
 }
 
@@ -173,9 +183,10 @@ __global__ void __launch_bounds__(kFgpX * kFgpY) k_fgp_iter(FgpArgs<T> A) {
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_fgp_final(FgpArgs<T> A, T* x) {
     const unsigned bx = blockIdx.x % A.gx, byz = blockIdx.x / A.gx;
-    const int i = bx * 64 + threadIdx.x, j = (byz % A.gy) * 4 + threadIdx.y, k = byz / A.gy;
+    const int ty = threadIdx.x / A.tw, i = bx * A.tw + (threadIdx.x - ty * A.tw);
+    const int j = (byz % A.gy) * A.th + ty, k = byz / A.gy;
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    if (i >= A.nx || j >= A.ny) return;
+    if (ty >= A.th || i >= A.nx || j >= A.ny) return;
     const size_t sy = (size_t)A.nx, sz = sy * A.ny, p = (size_t)k * sz + (size_t)j * sy + i;
     T v = 0;
     if (i >= 1) v += A.q[0][p - 1];
@@ -425,6 +436,45 @@ pat_status Ops<T>::reduce(int op, const pat_grid* g, long long n, const T* a, co
     return PAT_OK;
 }
 
+// tile and planes per CTA of k_fgp_iter; true: the tile compiled in
+template <typename T, int D> static bool fgp_tile(FgpArgs<T>& A) {
+    const auto up = [](int a, int b) { return (a + b - 1) / b; };
+    const int nsm = 152;
+    if (sizeof(T) == 4 && A.nx > 32) {
+        A.tw = kFgpX;
+        A.th = kFgpY;
+        A.gx = up(A.nx, A.tw);
+        A.gy = up(A.ny, A.th);
+        // a CTA reads one plane more than it writes, so long chunks save traffic as long as about four
+        // rounds of 4 CTAs per SM remain (13 planes at 256^3); at least 3 planes, or 2 where 3 would leave two
+        // CTAs per SM or less (128^3: 633 us with 3, 671 with 4, 708 with 2; 64^3: 270, 294, 247)
+        const long long planes = (long long)A.gx * A.gy * A.nz;
+        A.chunk = (int)std::max<long long>(planes < 6 * nsm ? 2 : 3, std::min<long long>(64, planes / (16 * nsm)));
+        return true;
+    }
+    // planes: the plane that is read but not written is dear where there are few (100^3 double: 2390 us with
+    // 4, 2560 with 2), CTAs are where the image is small (50 x 60 x 30: 460 us with 1, 740 with 2)
+    const double load = (double)A.nx * A.ny * A.nz / (nsm * 1024);   // points per SM, in 1024
+    A.chunk = D == 3 ? std::max(1, std::min({16, A.nz, (int)(load + 0.5), std::max(2, (int)(load / 2 + 0.5))})) : 1;
+    // sides: warps of the main tile count three times (x(r) and the update), those of its halo once, times the
+    // rounds of CTAs over the SMs.  Of all sides tried at 17 images in double this choice is on average 5 %
+    // slower than the best one, at most 20 % (40^3)
+    long long best = -1;
+    for (int tw : {up(A.nx, up(A.nx, 64)), std::min(A.nx, 32)})
+        for (int th = std::min({A.ny, kFgpRows, kFgpThreads / tw}); th >= 1 && (tw * th >= 64 || best < 0); --th) {
+            const int main = up(tw * th, 32), halo = up(tw + th, 32);   // warps
+            const long long n = (long long)up(A.nx, tw) * up(A.ny, th) * up(A.nz, A.chunk);
+            const long long cost = (n + nsm - 1) / nsm * (A.chunk * (3 * main + halo) + (D == 3 ? main : 0));
+            if (best >= 0 && cost >= best) continue;
+            best = cost;
+            A.tw = tw;
+            A.th = th;
+        }
+    A.gx = up(A.nx, A.tw);
+    A.gy = up(A.ny, A.th);
+    return false;
+}
+
 // the FGP loop: three rotating dual fields; every launch may start (programmatic dependent launch) while
 // its predecessor drains
 template <typename T, int D>
@@ -441,12 +491,7 @@ static pat_status fgp(const ImgDims& M, const T* z, T* x, double lam, int n_inne
     A.lam = (T)lam;
     A.step = (T)(1.0 / (4.0 * D * lam));
     A.nonneg = nonneg;
-    A.gx = (A.nx + kFgpX - 1) / kFgpX;
-    A.gy = (A.ny + kFgpY - 1) / kFgpY;
-    // planes per CTA: a CTA reads one plane more than it writes, so long chunks save traffic as long as
-    // about four rounds of 4 CTAs per SM remain (16 planes at 256^3); at least 4 planes
-    const long long want = 16LL * 152;
-    A.chunk = (int)std::max<long long>(4, std::min<long long>(64, (long long)A.gx * A.gy * A.nz / want));
+    const bool fixed = fgp_tile<T, D>(A);
     const unsigned gz = (D == 3) ? (A.nz + A.chunk - 1) / A.chunk : 1;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -468,19 +513,21 @@ static pat_status fgp(const ImgDims& M, const T* z, T* x, double lam, int n_inne
             for (int a = 0; a < D; ++a) A.qp[a] = A.q[a];
         A.w = (T)w;
         lc.gridDim = dim3(A.gx * A.gy * gz);
-        lc.blockDim = dim3(kFgpX, kFgpY);
+        lc.blockDim = dim3((std::max(A.tw * A.th, A.tw + A.th) + 31) / 32 * 32);   // a thread per halo point as well
         lc.numAttrs = it == 0 ? 0 : 1;   // the first launch follows the allocation and the caller's work
-        e = cudaLaunchKernelEx(&lc, k_fgp_iter<T, D>, A);
+        e = fixed ? cudaLaunchKernelEx(&lc, k_fgp_iter<T, D, true>, A) : cudaLaunchKernelEx(&lc, k_fgp_iter<T, D, false>, A);
         const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
         w = (t - 1.0) / tn;
         t = tn;
     }
     if (e == cudaSuccess) {
         for (int a = 0; a < D; ++a) A.q[a] = field(n_inner % 3, a);
-        A.gx = (A.nx + 63) / 64;
-        A.gy = (A.ny + 3) / 4;
+        A.tw = std::min(A.nx, 64);
+        A.th = std::min(A.ny, 256 / A.tw);
+        A.gx = (A.nx + A.tw - 1) / A.tw;
+        A.gy = (A.ny + A.th - 1) / A.th;
         lc.gridDim = dim3(A.gx * A.gy * (D == 3 ? A.nz : 1));
-        lc.blockDim = dim3(64, 4);
+        lc.blockDim = dim3((A.tw * A.th + 31) / 32 * 32);
         lc.numAttrs = 1;
         e = cudaLaunchKernelEx(&lc, k_fgp_final<T, D>, A, x);
     }
