@@ -244,8 +244,11 @@ pat_status pat_gradient_medium(pat_plan* plan, const void* p0, const void* resid
  *     k_c = k_cut * min over axes of pi / dx (0 < k_cut <= 1; 0.5 recommended).  compensate = 0 keeps
  *     the forward sign (no window, k_cut ignored).
  *   data  [Nt][Ns] measured data (host or device, plan precision); image [N] output.
- * The plan's smoothing switch is not applied.  Runs the per-phase kernels on the plan's own state
- * (the first call allocates a node map of N ints and (Nt + 1) Ns values, kept by the plan). */
+ * The plan's smoothing switch is not applied.  Runs on the plan's own state: 2-D plans on path 1 or 2 in
+ * one persistent launch (axes with a mixed-radix schedule: all but a few long ones), whose bounded wait
+ * pat_plan_status reports, other plans in the per-phase kernels.  The first call allocates a node map of
+ * N ints and (Nt + 1) Ns values, and for absorbing plans with mixed-radix y / z passes two tables of
+ * multipliers on the half spectrum; the plan keeps them. */
 pat_status pat_time_reversal(pat_plan* plan, const void* data, void* image, int compensate, double k_cut,
                              void* stream);
 

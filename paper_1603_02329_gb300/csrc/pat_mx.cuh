@@ -579,7 +579,9 @@ template <typename T> __global__ void k_mx_kap(MxTableArgs A, T* kap, T* abs) {
     }
 }
 
-// grid (fields or 1, column tiles, outer lines): one field per CTA for the plain and field-wise modes
+// grid (fields or 1, column tiles, outer lines): one field per CTA for the plain and field-wise modes.  The
+// register bound (80 in FP32, 128 in double) keeps three and two CTAs of 256 threads per SM; only GRADT, which
+// holds two spectra, spills under it (FP32 444 bytes stored, 464 loaded in 3-D; double 496 and 496).
 template <typename T, int D, int MODE>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_mx_spec(DevPlan<T> P, MxAxis x, const cplx<T>* __restrict__ tw, int W, int lgW,
                                                  int lax, const T* __restrict__ mt) {
